@@ -219,6 +219,13 @@ ProjArgs proj_args_cropped(const xcf_geometry *g, const Crop &c, int interp) {
     return a;
 }
 
+// the same for a library's own templates: bilinear lookups read its 2 x 2 cells
+ProjArgs proj_args_of(const xcf_library *lib, const Crop &c, int interp) {
+    ProjArgs a = proj_args_cropped(&lib->geom, c, interp);
+    a.quad = lib->quad;
+    return a;
+}
+
 PrepArgs prep_args_square(const Crop &c, const Resolved &r) {
     PrepArgs a;
     a.N = c.n;
@@ -373,7 +380,7 @@ int refine_chunk(xcf_ctx *ctx, const xcf_library *lib, const float *patterns, in
     if ((rc = scratch_t(ctx, S_ACTIVE, P, &active))) return rc;
     if ((rc = scratch_t(ctx, S_Q1, (size_t)P * 4, &q1))) return rc;
     const PrepArgs pa = prep_args(g, c, r), ps = prep_args_square(c, r);
-    const ProjArgs pj = proj_args_cropped(g, c, ctx->opt.master_interp);
+    const ProjArgs pj = proj_args_of(lib, c, ctx->opt.master_interp);
     const double alpha = alpha_of(g);
     if (!patterns_ready)   // else sp, yp, degen already hold this chunk's patterns
         XCF_LAUNCH(XCF_STAGE_PREP, st, run_prep(ctx,patterns, P, pa, sp, yp, degen, nullptr, st), "prep patterns");
@@ -577,6 +584,35 @@ int xcf_build_library_images(xcf_ctx *ctx, const float *images, const double *qu
 }
 
 namespace {
+// The library's own copies of the orientations and the master, in one
+// allocation with the master's 2 x 2 cells.  The cells are kept for masters up
+// to half the 129 MB L2 (M <= 1,448), where they stay resident beside the
+// spectra; a larger master, or one whose cells find no memory (32 M^2 bytes),
+// is read as it is.
+constexpr size_t kQuadMaxBytes = (size_t)64 << 20;
+cudaError_t library_head(xcf_library *lib, const double *quats, const float *master, cudaStream_t st) {
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t mm = 2 * (size_t)lib->M * lib->M, qb = up(sizeof(double) * 4 * lib->T);
+    const size_t mb = master ? up(sizeof(float) * mm) : 0;
+    size_t quad = master && sizeof(float4) * mm <= kQuadMaxBytes ? sizeof(float4) * mm : 0;
+    cudaError_t e = cudaMalloc(&lib->head, qb + mb + quad);
+    if (e != cudaSuccess && quad) {
+        cudaGetLastError();
+        quad = 0;
+        e = cudaMalloc(&lib->head, qb + mb);
+    }
+    if (e != cudaSuccess) return e;
+    char *base = static_cast<char *>(lib->head);
+    lib->quats = reinterpret_cast<double *>(base);
+    e = cudaMemcpyAsync(lib->quats, quats, sizeof(double) * 4 * lib->T, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess || !master) return e;
+    lib->master = reinterpret_cast<float *>(base + qb);
+    e = cudaMemcpyAsync(lib->master, master, sizeof(float) * mm, cudaMemcpyDeviceToDevice, st);
+    if (e != cudaSuccess || !quad) return e;
+    lib->quad = reinterpret_cast<float4 *>(base + qb + mb);
+    return launch_master_quads(lib->master, lib->M, lib->quad, st);
+}
+
 // spectra == false: the library keeps its orientations, master and geometry
 // but no FFT spectra (an NDP-only library)
 int build_from_master(xcf_ctx *ctx, const float *master, int32_t M, const double *quats, int32_t T,
@@ -604,18 +640,14 @@ int build_from_master(xcf_ctx *ctx, const float *master, int32_t M, const double
     memcpy(lib->pc, c.pc, sizeof c.pc);
     const size_t H = (size_t)c.n * (c.n / 2 + 1);
     cudaError_t e = spectra ? cudaMalloc(&lib->spectra, sizeof(float2) * H * T) : cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&lib->quats, sizeof(double) * 4 * T);
-    if (e == cudaSuccess) e = cudaMalloc(&lib->master, sizeof(float) * 2 * (size_t)M * M);
-    if (e != cudaSuccess) {
+    if (e == cudaSuccess) e = library_head(lib, quats, master, st);
+    if (!lib->head) {
         cudaGetLastError();
         xcf_library_free(lib);
         return fail(ctx, XCF_ERR_OOM, "xcf_build_library: allocation failed");
     }
-    e = cudaMemcpyAsync(lib->quats, quats, sizeof(double) * 4 * T, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(lib->master, master, sizeof(float) * 2 * (size_t)M * M, cudaMemcpyDeviceToDevice, st);
     // project and pre-process in chunks (bounded image scratch)
-    const ProjArgs pj = proj_args_cropped(g, c, ctx->opt.master_interp);
+    const ProjArgs pj = proj_args_of(lib, c, ctx->opt.master_interp);
     const PrepArgs ps = prep_args_square(c, r);
     int *degen = nullptr;
     float *img = nullptr;
@@ -679,16 +711,12 @@ int build_from_images(xcf_ctx *ctx, const float *images, const double *quats, in
     memcpy(lib->pc, c.pc, sizeof c.pc);
     const size_t H = (size_t)c.n * (c.n / 2 + 1);
     cudaError_t e = spectra ? cudaMalloc(&lib->spectra, sizeof(float2) * H * T) : cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&lib->quats, sizeof(double) * 4 * T);
-    if (e == cudaSuccess && master) e = cudaMalloc(&lib->master, sizeof(float) * 2 * (size_t)M * M);
-    if (e != cudaSuccess) {
+    if (e == cudaSuccess) e = library_head(lib, quats, master, st);
+    if (!lib->head) {
         cudaGetLastError();
         xcf_library_free(lib);
         return fail(ctx, XCF_ERR_OOM, "xcf_build_library_images: allocation failed");
     }
-    e = cudaMemcpyAsync(lib->quats, quats, sizeof(double) * 4 * T, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess && master)
-        e = cudaMemcpyAsync(lib->master, master, sizeof(float) * 2 * (size_t)M * M, cudaMemcpyDeviceToDevice, st);
     int *degen = nullptr;
     if ((rc = scratch_t(ctx, S_DEGEN, T, &degen))) {
         xcf_library_free(lib);
@@ -721,8 +749,7 @@ int xcf_library_free(xcf_library *lib) {
     if (lib->spectra_pk) cudaFree(lib->spectra_pk);
     if (lib->bf16) cudaFree(lib->bf16);
     if (lib->ndp32) cudaFree(lib->ndp32);
-    if (lib->quats) cudaFree(lib->quats);
-    if (lib->master) cudaFree(lib->master);
+    if (lib->head) cudaFree(lib->head);
     delete lib;
     return XCF_OK;
 }
@@ -1082,7 +1109,7 @@ int make_screen_images(xcf_ctx *ctx, xcf_library *lib, const float *images, cuda
             if ((rc = scratch_t(ctx, S_IMG, nn * nt, &img))) return rc;
             XCF_LAUNCH(XCF_STAGE_PROJECT, st,
                        launch_project(lib->master, lib->M, lib->quats + 4 * (size_t)t0, nullptr, nullptr, nt,
-                                      proj_args_cropped(g, c, ctx->opt.master_interp), img, st),
+                                      proj_args_of(lib, c, ctx->opt.master_interp), img, st),
                        "screen project");
             XCF_LAUNCH(XCF_STAGE_PREP, st,
                        run_prep(ctx, img, nt, prep_args_square(c, r), spec, spat, degen, nullptr, st), "screen prep");
@@ -1122,7 +1149,7 @@ int make_ndp_images(xcf_ctx *ctx, xcf_library *lib, const float *images, cudaStr
             if ((rc = scratch_t(ctx, S_IMG, nn * nt, &img))) return rc;
             XCF_LAUNCH(XCF_STAGE_PROJECT, st,
                        launch_project(lib->master, lib->M, lib->quats + 4 * (size_t)t0, nullptr, nullptr, nt,
-                                      proj_args_cropped(g, c, ctx->opt.master_interp), img, st),
+                                      proj_args_of(lib, c, ctx->opt.master_interp), img, st),
                        "ndp project");
             if ((rc = ndp_operands(ctx, img, nt, (long)nn, c.n, 0, 0, c.n, o32, o16, nullptr, st))) return rc;
         }
@@ -1768,7 +1795,7 @@ int xcf_index_learned(xcf_ctx *ctx, xcf_net *net, const xcf_library *lib, const 
     const Resolved r = resolve(ctx->opt, c.n);
     const int n = c.n, H = n * (n / 2 + 1), k = net->k;
     const size_t img = (size_t)g->width * g->height;
-    const ProjArgs pj = proj_args_cropped(g, c, ctx->opt.master_interp);
+    const ProjArgs pj = proj_args_of(lib, c, ctx->opt.master_interp);
     const PrepArgs pa = prep_args(g, c, r), ps = prep_args_square(c, r);
     for (int p0 = 0; p0 < P; p0 += kChunk) {
         const int np = P - p0 < kChunk ? P - p0 : kChunk;

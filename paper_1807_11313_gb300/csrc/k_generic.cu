@@ -50,8 +50,8 @@ template <int N>
 __host__ __device__ constexpr int search_threads() { return N >= 128 ? 1024 : kThreads; }
 
 // PROJ: the image is projected from the master pattern (ps) while it is
-// loaded, instead of read from img
-template <int N, int PT = prep_threads<N>(), bool PROJ = false>
+// loaded, instead of read from img (QUAD: from the master's 2 x 2 cells)
+template <int N, bool PROJ = false, bool QUAD = false, int PT = prep_threads<N>()>
 __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img, PrepArgs a,
                                                         float2 *__restrict__ spec, float *__restrict__ spatial,
                                                         int *__restrict__ degen, const int *__restrict__ active,
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
     }
     auto pixel = [&](int r, int c) -> float {   // image pixel (a.oy + r, a.ox + c)
         if constexpr (PROJ)
-            return proj::pixel(f, ps.master, ps.M, ps.a, a.oy + r, a.ox + c);
+            return proj::pixel<QUAD>(f, ps.master, ps.M, ps.a, a.oy + r, a.ox + c);
         else
             return src[(size_t)(a.oy + r) * a.W + a.ox + c];
     };
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
         // every pixel of this thread lies in column tid mod N: its column part once
         const int c = tid % N;
         const proj::Col col = proj::column(f, ps.a, a.ox + c);
-        for (int r = tid / N; r < N; r += PT / N) take(r, c, proj::pixel(f, col, ps.master, ps.M, ps.a, a.oy + r));
+        for (int r = tid / N; r < N; r += PT / N) take(r, c, proj::pixel<QUAD>(f, col, ps.master, ps.M, ps.a, a.oy + r));
     } else {
         for (int idx = tid; idx < N * N; idx += PT) {
             const int r = idx / N, c = idx % N;
@@ -602,7 +602,7 @@ template <int N>
 cudaError_t prep_projected_n(const ProjSrc &src, int P, const PrepArgs &a, float2 *spec, float *spatial, int *degen,
                              const int *active, cudaStream_t st) {
     const size_t sm = smem_prep_real<N>();
-    auto *k = k_prep_real<N, prep_threads<N>(), true>;
+    auto *k = proj::use_quad(src.a) ? k_prep_real<N, true, true> : k_prep_real<N, true, false>;
     cudaError_t e = set_smem(k, sm);
     if (e != cudaSuccess) return e;
     k<<<P, prep_threads<N>(), sm, st>>>(nullptr, a, spec, spatial, degen, active, src);

@@ -20,6 +20,7 @@ struct ProjArgs {
     double alpha;             // detector -> sample rotation about x, radians
     int interp = 0;           // master lookup: 0 bilinear, 1 bicubic (Keys)
     double ca = 1.0, sa = 0.0;   // cos / sin of alpha (set by launch_project)
+    const float4 *quad = nullptr;   // bilinear lookups: the master as 2 x 2 cells (launch_master_quads), or null
 };
 
 // pre-processing: images [P, H, W] -> half spectra [P, N, N/2+1] (+ spatial [P, N, N])
@@ -138,6 +139,10 @@ cudaError_t launch_keys_to_best(const unsigned long long *keys, int P, int *best
 
 cudaError_t launch_project(const float *master, int M, const double *quats, const double *pcs,
                            const int *active, int P, const ProjArgs &a, float *out, cudaStream_t st);
+
+// the master [2][M][M] as one 16-byte element per cell corner (i, j): values
+// (i, j), (i + 1, j), (i, j + 1), (i + 1, j + 1), edges repeated -> quad [2][M][M]
+cudaError_t launch_master_quads(const float *master, int M, float4 *quad, cudaStream_t st);
 
 cudaError_t launch_logpolar(const float *spatial, const int *active, int P, int N, int nr, int neta,
                             float rmin, float rmax, float *out, cudaStream_t st);
