@@ -1,5 +1,6 @@
-// Pre-processing, the all-sides search kernel and the single-surface peak
-// kernel for N in {16, 32, 64, 96, 128, 160}.  The search and peak kernels
+// Pre-processing (N in {16, 32, 64, 96, 160}; 128 in k_prep128.cu), the
+// all-sides search kernel and the single-surface peak kernel for N in {16, 32,
+// 64, 96, 128, 160}.  The search and peak kernels
 // hold one N x N complex array in shared memory (rows padded to N + 1) and
 // transform its lines with the warp line FFT (registers and shuffles for
 // N = R x 32 >= 64, mixed radix at 96 and 160; radix-2 butterflies spread
@@ -24,9 +25,8 @@ using namespace gen;
 // then split by Hermitian symmetry into R[y][0..N/2]); the columns of R are
 // transformed as their even- and odd-row halves (N/2-point transforms) joined
 // by one radix-2 stage.  Bins 0 and N/2 of every row are real, so they share
-// one complex slot per row pair.  The N/2 x (N+1) complex array (66 KB at
-// N = 128) lets three CTAs share an SM.  The spatial output runs the same
-// steps backwards.
+// one complex slot per row pair.  The spatial output runs the same steps
+// backwards.
 // layout of buf after the row split, row pr (image rows 2pr, 2pr+1):
 //   [0]        (Ra[0], Ra[N/2])   real bins of row 2pr
 //   [1, N/2)   Ra[v]
@@ -43,15 +43,13 @@ constexpr size_t smem_prep_real() {
 // threads per CTA: more warps for the larger sides hide the shared-memory and
 // global-load latency of the line transforms
 template <int N>
-constexpr int prep_threads() { return N >= 128 ? 512 : kThreads; }
-template <int N>
 constexpr int peak_threads() { return N >= 128 ? 1024 : kThreads; }
 template <int N>
 __host__ __device__ constexpr int search_threads() { return N >= 128 ? 1024 : kThreads; }
 
 // PROJ: the image is projected from the master pattern (ps) while it is
 // loaded, instead of read from img (QUAD: from the master's 2 x 2 cells)
-template <int N, bool PROJ = false, bool QUAD = false, int PT = prep_threads<N>()>
+template <int N, bool PROJ = false, bool QUAD = false, int PT = kThreads>
 __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img, PrepArgs a,
                                                         float2 *__restrict__ spec, float *__restrict__ spatial,
                                                         int *__restrict__ degen, const int *__restrict__ active,
@@ -594,7 +592,7 @@ cudaError_t prep_n(const float *img, int P, const PrepArgs &a, float2 *spec, flo
     const size_t sm = smem_prep_real<N>();
     cudaError_t e = set_smem(k_prep_real<N>, sm);
     if (e != cudaSuccess) return e;
-    k_prep_real<N><<<P, prep_threads<N>(), sm, st>>>(img, a, spec, spatial, degen, active, ProjSrc{});
+    k_prep_real<N><<<P, kThreads, sm, st>>>(img, a, spec, spatial, degen, active, ProjSrc{});
     return cudaGetLastError();
 }
 
@@ -605,7 +603,7 @@ cudaError_t prep_projected_n(const ProjSrc &src, int P, const PrepArgs &a, float
     auto *k = proj::use_quad(src.a) ? k_prep_real<N, true, true> : k_prep_real<N, true, false>;
     cudaError_t e = set_smem(k, sm);
     if (e != cudaSuccess) return e;
-    k<<<P, prep_threads<N>(), sm, st>>>(nullptr, a, spec, spatial, degen, active, src);
+    k<<<P, kThreads, sm, st>>>(nullptr, a, spec, spatial, degen, active, src);
     return cudaGetLastError();
 }
 
@@ -672,7 +670,7 @@ cudaError_t launch_prep(const float *img, int P, const PrepArgs &a, float2 *spec
         case 16: return prep_n<16>(img, P, a, spec, spatial, degen, active, st);
         case 32: return prep_n<32>(img, P, a, spec, spatial, degen, active, st);
         case 64: return prep_n<64>(img, P, a, spec, spatial, degen, active, st);
-        case 128: return prep_n<128>(img, P, a, spec, spatial, degen, active, st);
+        case 128: return launch_prep128(img, P, a, spec, spatial, degen, active, st);
         case 96: return prep_cplx_n<96>(img, P, a, spec, spatial, degen, active, st);
         case 160: return prep_cplx_n<160>(img, P, a, spec, spatial, degen, active, st);
         case 200: return launch_prep_n200(img, P, a, spec, spatial, degen, active, st);
@@ -691,7 +689,7 @@ cudaError_t launch_prep_projected(const ProjSrc &src, int P, const PrepArgs &a, 
         case 16: return prep_projected_n<16>(s, P, a, spec, spatial, degen, active, st);
         case 32: return prep_projected_n<32>(s, P, a, spec, spatial, degen, active, st);
         case 64: return prep_projected_n<64>(s, P, a, spec, spatial, degen, active, st);
-        case 128: return prep_projected_n<128>(s, P, a, spec, spatial, degen, active, st);
+        case 128: return launch_prep128_projected(s, P, a, spec, spatial, degen, active, st);
         default: return cudaErrorNotSupported;
     }
 }

@@ -43,6 +43,12 @@ struct ProjSrc {
 cudaError_t launch_prep_projected(const ProjSrc &src, int P, const PrepArgs &a, float2 *spec, float *spatial,
                                   int *degen, const int *active, cudaStream_t st);
 
+// N = 128 (k_prep128.cu): the two launchers above for that side
+cudaError_t launch_prep128(const float *img, int P, const PrepArgs &a, float2 *spec, float *spatial, int *degen,
+                           const int *active, cudaStream_t st);
+cudaError_t launch_prep128_projected(const ProjSrc &src, int P, const PrepArgs &a, float2 *spec, float *spatial,
+                                     int *degen, const int *active, cudaStream_t st);
+
 // all-pairs search: per-pattern best key (atomicMax) and optional per-pair peaks [P, T]
 cudaError_t launch_search(int N, const float2 *St, int T, const float2 *Sp, const int *degen, int P,
                           unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st);
