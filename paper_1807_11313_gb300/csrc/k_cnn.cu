@@ -11,11 +11,10 @@
 // 256 -> 6k; head h turns (a1, a2) into R = [b1 b2 b3] by Gram-Schmidt (the
 // continuous 6-D representation of Zhou et al. 2019).
 //
-// Every layer is a tiled FP32 matrix product whose operand loaders gather
-// from the activations directly (implicit im2col), so no unfolded copy is
-// written: C[m][n] = sum_k A(m, k) B(k, n) with the layer's loaders and
-// epilogue.  Weight gradients split the long reduction over gridDim.z and
-// accumulate with atomics.
+// The FP32 convolutions are in k_conv32.cu, the BF16 ones in k_conv.cu.  The fc
+// layers are small tiled FP32 matrix products C[m][n] = sum_k A(m, k) B(k, n)
+// with a layer's loaders and epilogue; their weight gradients split the
+// reduction over gridDim.z and sum the partials in order.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -25,7 +24,11 @@
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, GT = 256;
+// 32 x 32 tiles, 32 deep: the fc layers' products (256 x B x 128 and the like)
+// are a few us of latency each, so they take many small CTAs and few slices
+// (64 x 64 x 16 tiles: 12-31 us per layer at B = 256)
+constexpr int BM = 32, BN = 32, BK = 32, GT = 256;
+constexpr int GM = BM / 16, GN = BN / 16;   // outputs per thread
 
 template <class LA, class LB, class EP>
 __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, int kper, LA la, LB lb, EP ep) {
@@ -34,10 +37,10 @@ __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, int kper, LA l
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
     const int kb = blockIdx.z * kper, ke = min(K, kb + kper);
-    float acc[4][4] = {};
+    float acc[GM][GN] = {};
     for (int k0 = kb; k0 < ke; k0 += BK) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < BM * BK / GT; ++i) {
             const int e = tid + i * GT;
             const int am = e / BK, ak = e % BK;       // A: consecutive threads walk k
             const int m = m0 + am, k = k0 + ak;
@@ -49,24 +52,23 @@ __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, int kper, LA l
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float a[4], b[4];
+            float a[GM], b[GN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[kk][ty * 4 + i];
-                b[i] = Bs[kk][tx * 4 + i];
-            }
+            for (int i = 0; i < GM; ++i) a[i] = As[kk][ty * GM + i];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < GN; ++j) b[j] = Bs[kk][tx * GN + j];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < GM; ++i)
+#pragma unroll
+                for (int j = 0; j < GN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < GM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
+        for (int j = 0; j < GN; ++j) {
+            const int m = m0 + ty * GM + i, n = n0 + tx * GN + j;
             if (m < M && n < N) ep(m, n, acc[i][j]);
         }
 }
@@ -99,28 +101,7 @@ int grad_splits(int M, int N, int K, int num_sms) {
 }
 
 // ------------------------------------------------------------- loaders
-struct Src {   // layer input: activations [B][C][S][S], or the raw patterns (layer 1)
-    const float *x;
-    int C, S;
-    long img_stride, row_stride;   // floats between images / rows
-    int ox, oy;                    // crop offsets (layer 1)
-    const float2 *affine;          // per-image (scale, shift) of the standardisation, or null
-};
-
-// im2col element (k = ci*9 + ky*3 + kx, n = b*So*So + oy*So + ox)
-__device__ __forceinline__ float im2col(const Src &s, int So, int k, int n) {
-    const int ci = k / 9, r = k - ci * 9, ky = r / 3, kx = r - ky * 3;
-    const int lg = __ffs(So) - 1;   // output sides are powers of two: shifts, not divisions
-    const int b = n >> (2 * lg), p = n & (So * So - 1), oy = p >> lg, ox = p & (So - 1);
-    const int iy = 2 * oy - 1 + ky, ix = 2 * ox - 1 + kx;
-    if (iy < 0 || iy >= s.S || ix < 0 || ix >= s.S) return 0.f;
-    const float v = s.x[b * s.img_stride + (long)ci * s.S * s.S + (long)(s.oy + iy) * s.row_stride + s.ox + ix];
-    if (!s.affine) return v;
-    const float2 a = s.affine[b];
-    return fmaf(v, a.x, a.y);
-}
-
-struct LoadW {   // weights [M][K] row-major (conv W[co][ci*9] or fc W[out][in])
+struct LoadW {   // weights [M][K] row-major (W[out][in])
     const float *w;
     int K;
     __device__ float operator()(int m, int k) const { return w[(long)m * K + k]; }
@@ -129,49 +110,6 @@ struct LoadWT {   // transposed weights: A(m, k) = W[k][m] of a [K][M] matrix
     const float *w;
     int M;
     __device__ float operator()(int m, int k) const { return w[(long)k * M + m]; }
-};
-struct LoadWconvT {   // A(m = ci, k = co*9 + r) = W[co][ci][r] of conv weights [Co][Ci][9]
-    const float *w;
-    int Ci;
-    __device__ float operator()(int m, int k) const {
-        const int co = k / 9, r = k - co * 9;
-        return w[((long)co * Ci + m) * 9 + r];
-    }
-};
-struct LoadIm2col {
-    Src s;
-    int So;
-    __device__ float operator()(int k, int n) const { return im2col(s, So, k, n); }
-};
-struct LoadIm2colT {   // B(k = (b, p), n = ci*9 + ...) for the weight gradient
-    Src s;
-    int So;
-    __device__ float operator()(int k, int n) const { return im2col(s, So, n, k); }
-};
-struct LoadGradT {   // A(m = co, k = (b, p)) = g[b][co][p]
-    const float *g;
-    int C, Q;
-    __device__ float operator()(int m, int k) const {
-        const int b = k >> (__ffs(Q) - 1), p = k & (Q - 1);   // Q is a power of two
-        return g[((long)b * C + m) * Q + p];
-    }
-};
-// dX gather: B(k = co*9 + ky*3 + kx, n = b*Si*Si + iy*Si + ix) = g[b][co][oy][ox]
-// where iy = 2 oy - 1 + ky (zero where no such output exists)
-struct LoadGradScatter {
-    const float *g;
-    int Co, So;
-    __device__ float operator()(int k, int n) const {
-        const int Si = 2 * So;
-        const int co = k / 9, r = k - co * 9, ky = r / 3, kx = r - ky * 3;
-        const int lg = __ffs(Si) - 1;   // a power of two
-        const int b = n >> (2 * lg), p = n & (Si * Si - 1), iy = p >> lg, ix = p & (Si - 1);
-        const int ty = iy + 1 - ky, tx = ix + 1 - kx;
-        if (ty < 0 || tx < 0 || (ty & 1) || (tx & 1)) return 0.f;
-        const int oy = ty >> 1, ox = tx >> 1;
-        if (oy >= So || ox >= So) return 0.f;
-        return g[(((long)b * Co + co) * So + oy) * So + ox];
-    }
 };
 struct LoadRows {   // B(k, n) = X[n][k] of a row-major [N][K] matrix (a batch of vectors)
     const float *x;
@@ -190,15 +128,6 @@ struct LoadRowsB {   // B(k, n) = X[k][n] of a row-major [K][N] matrix
 };
 
 // ----------------------------------------------------------- epilogues
-struct EpConv {   // y[b][co][p] = relu(acc + bias[co])
-    float *y;
-    const float *bias;
-    int Co, Q;
-    __device__ void operator()(int m, int n, float v) const {
-        const int b = n >> (__ffs(Q) - 1), p = n & (Q - 1);   // Q is a power of two
-        y[((long)b * Co + m) * Q + p] = fmaxf(v + bias[m], 0.f);
-    }
-};
 struct EpVec {   // y[n][m] = act(acc + bias[m]) for a batch of vectors
     float *y;
     const float *bias;
@@ -215,16 +144,6 @@ struct EpMasked {   // y[n][m] = acc * (mask[n][m] > 0) (gradient through a ReLU
     int M;
     __device__ void operator()(int m, int n, float v) const {
         const long i = (long)n * M + m;
-        y[i] = mask[i] > 0.f ? v : 0.f;
-    }
-};
-struct EpMaskedImg {   // gx[b][ci][p] = acc * (a[b][ci][p] > 0), n = b*Q + p
-    float *y;
-    const float *mask;
-    int C, Q;
-    __device__ void operator()(int m, int n, float v) const {
-        const int b = n >> (__ffs(Q) - 1), p = n & (Q - 1);   // Q is a power of two
-        const long i = ((long)b * C + m) * Q + p;
         y[i] = mask[i] > 0.f ? v : 0.f;
     }
 };
@@ -461,76 +380,108 @@ __device__ M3 cubic_op(int s) {
     return {{1, 0, 0, 0, 1, 0, 0, 0, 1}};
 }
 
-// one thread per pattern: winner-takes-all loss over heads and cubic operators
-__global__ void k_cnn_head_loss(const float *__restrict__ out, int B, int k, const double *__restrict__ qgt,
-                                float *__restrict__ gout, double *__restrict__ loss_sum, int *__restrict__ winners) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+// one warp per pattern: winner-takes-all loss over heads and cubic operators.
+// The FP64 pipe is narrow, so the k x 24 candidates are spread over the lanes
+// (one thread per pattern: 404 us at B = 256, k = 8, on two SMs), and an
+// operator, a signed permutation, takes rows of Rg instead of products.
+constexpr int kLossWarps = 4;
+__global__ void __launch_bounds__(32 * kLossWarps) k_cnn_head_loss(const float *__restrict__ out, int B, int k,
+                                                                   const double *__restrict__ qgt,
+                                                                   float *__restrict__ gout,
+                                                                   double *__restrict__ loss_sum,
+                                                                   int *__restrict__ winners) {
+    __shared__ double part[kLossWarps];
+    __shared__ signed char op_row[24][3], op_sign[24][3];   // row i of operator s: sign times row op_row of Rg
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x * kLossWarps + warp;
+    if (threadIdx.x < 24) {
+        const M3 S = cubic_op(threadIdx.x);
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j)
+                if (S.a[3 * i + j] != 0.0) {
+                    op_row[threadIdx.x][i] = (signed char)j;
+                    op_sign[threadIdx.x][i] = S.a[3 * i + j] > 0.0 ? 1 : -1;
+                }
+    }
+    __syncthreads();
     double my = 0.0;
-    if (b < B) {
+    if (b < B) {   // uniform over the warp
         const M3 Rg = quat_matrix(qgt + 4 * b);
         double best = 1e300;
-        int bh = 0, bs = 0;
-        for (int h = 0; h < k; ++h) {
+        int be = 0x7fffffff;   // head * 24 + operator of the lane's best; the lowest among equals
+        for (int e = lane; e < k * 24; e += 32) {
+            const int h = e / 24, s = e - h * 24;
             double b1[3], b2[3], b3[3], n1, n2, d;
             gs(out + ((long)b * k + h) * 6, b1, b2, b3, &n1, &n2, &d);
-            for (int s = 0; s < 24; ++s) {
-                const M3 S = cubic_op(s);
-                double l = 0.0;
-                for (int i = 0; i < 3; ++i)
-                    for (int j = 0; j < 3; ++j) {
-                        const double t = S.a[i * 3] * Rg.a[j] + S.a[i * 3 + 1] * Rg.a[3 + j] + S.a[i * 3 + 2] * Rg.a[6 + j];
-                        const double r = j == 0 ? b1[i] : (j == 1 ? b2[i] : b3[i]);
-                        l += (r - t) * (r - t);
-                    }
-                if (l < best) {
-                    best = l;
-                    bh = h;
-                    bs = s;
+            double l = 0.0;
+            for (int i = 0; i < 3; ++i) {
+                const int row = op_row[s][i];
+                const double sg = op_sign[s][i];
+                for (int j = 0; j < 3; ++j) {
+                    const double t = sg * (row == 0 ? Rg.a[j] : row == 1 ? Rg.a[3 + j] : Rg.a[6 + j]);
+                    const double r = j == 0 ? b1[i] : (j == 1 ? b2[i] : b3[i]);
+                    l += (r - t) * (r - t);
                 }
             }
-        }
-        my = best / B;
-        if (winners) {
-            winners[2 * b] = bh;
-            winners[2 * b + 1] = bs;
-        }
-        // gradient of |R - S Rg|^2 through Gram-Schmidt, scaled by 1/B
-        double b1[3], b2[3], b3[3], n1, n2, d;
-        const float *a = out + ((long)b * k + bh) * 6;
-        gs(a, b1, b2, b3, &n1, &n2, &d);
-        const M3 S = cubic_op(bs);
-        double g1[3], g2[3], g3[3];
-        for (int i = 0; i < 3; ++i) {
-            double t[3];
-            for (int j = 0; j < 3; ++j)
-                t[j] = S.a[i * 3] * Rg.a[j] + S.a[i * 3 + 1] * Rg.a[3 + j] + S.a[i * 3 + 2] * Rg.a[6 + j];
-            g1[i] = 2.0 * (b1[i] - t[0]) / B;
-            g2[i] = 2.0 * (b2[i] - t[1]) / B;
-            g3[i] = 2.0 * (b3[i] - t[2]) / B;
-        }
-        double gb1[3], gb2[3], t[3], gu[3], ga1[3], ga2[3];
-        cross(b2, g3, t);
-        for (int i = 0; i < 3; ++i) gb1[i] = g1[i] + t[i];
-        cross(g3, b1, t);
-        for (int i = 0; i < 3; ++i) gb2[i] = g2[i] + t[i];
-        const double pb2 = dot(b2, gb2);
-        for (int i = 0; i < 3; ++i) gu[i] = (gb2[i] - pb2 * b2[i]) / n2;
-        const double pu = dot(b1, gu);
-        for (int i = 0; i < 3; ++i) {
-            ga2[i] = gu[i] - pu * b1[i];
-            gb1[i] += -pu * a[3 + i] - d * gu[i];
-        }
-        const double pb1 = dot(b1, gb1);
-        for (int i = 0; i < 3; ++i) ga1[i] = (gb1[i] - pb1 * b1[i]) / n1;
-        for (int h = 0; h < k; ++h)
-            for (int i = 0; i < 6; ++i) {
-                double v = 0.0;
-                if (h == bh) v = i < 3 ? ga1[i] : ga2[i - 3];
-                gout[((long)b * k + h) * 6 + i] = (float)v;
+            if (l < best) {
+                best = l;
+                be = e;
             }
+        }
+        for (int o = 16; o; o >>= 1) {
+            const double ol = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oe = __shfl_xor_sync(0xffffffffu, be, o);
+            if (ol < best || (ol == best && oe < be)) {
+                best = ol;
+                be = oe;
+            }
+        }
+        const int bh = be == 0x7fffffff ? 0 : be / 24, bs = be == 0x7fffffff ? 0 : be - bh * 24;
+        for (int i = lane; i < 6 * k; i += 32)
+            if (i / 6 != bh) gout[(long)b * k * 6 + i] = 0.f;
+        if (lane == 0) {
+            my = best / B;
+            if (winners) {
+                winners[2 * b] = bh;
+                winners[2 * b + 1] = bs;
+            }
+            // gradient of |R - S Rg|^2 through Gram-Schmidt, scaled by 1/B
+            double b1[3], b2[3], b3[3], n1, n2, d;
+            const float *a = out + ((long)b * k + bh) * 6;
+            gs(a, b1, b2, b3, &n1, &n2, &d);
+            const M3 S = cubic_op(bs);
+            double g1[3], g2[3], g3[3];
+            for (int i = 0; i < 3; ++i) {
+                double t[3];
+                for (int j = 0; j < 3; ++j)
+                    t[j] = S.a[i * 3] * Rg.a[j] + S.a[i * 3 + 1] * Rg.a[3 + j] + S.a[i * 3 + 2] * Rg.a[6 + j];
+                g1[i] = 2.0 * (b1[i] - t[0]) / B;
+                g2[i] = 2.0 * (b2[i] - t[1]) / B;
+                g3[i] = 2.0 * (b3[i] - t[2]) / B;
+            }
+            double gb1[3], gb2[3], t[3], gu[3], ga1[3], ga2[3];
+            cross(b2, g3, t);
+            for (int i = 0; i < 3; ++i) gb1[i] = g1[i] + t[i];
+            cross(g3, b1, t);
+            for (int i = 0; i < 3; ++i) gb2[i] = g2[i] + t[i];
+            const double pb2 = dot(b2, gb2);
+            for (int i = 0; i < 3; ++i) gu[i] = (gb2[i] - pb2 * b2[i]) / n2;
+            const double pu = dot(b1, gu);
+            for (int i = 0; i < 3; ++i) {
+                ga2[i] = gu[i] - pu * b1[i];
+                gb1[i] += -pu * a[3 + i] - d * gu[i];
+            }
+            const double pb1 = dot(b1, gb1);
+            for (int i = 0; i < 3; ++i) ga1[i] = (gb1[i] - pb1 * b1[i]) / n1;
+            for (int i = 0; i < 6; ++i) gout[((long)b * k + bh) * 6 + i] = (float)(i < 3 ? ga1[i] : ga2[i - 3]);
+        }
     }
-    for (int o = 16; o; o >>= 1) my += __shfl_xor_sync(0xffffffffu, my, o);
-    if ((threadIdx.x & 31) == 0 && loss_sum) atomicAdd(loss_sum, my);
+    if (lane == 0) part[warp] = my;
+    __syncthreads();
+    if (threadIdx.x == 0 && loss_sum) {
+        double t = 0.0;
+        for (int w = 0; w < kLossWarps; ++w) t += part[w];
+        atomicAdd(loss_sum, t);
+    }
 }
 
 // proposals: quaternion (w >= 0) of the Gram-Schmidt rotation of every head
@@ -723,9 +674,12 @@ constexpr size_t kPartFloats = (size_t)1 << 22;
 constexpr int kBiasRows = 64;
 constexpr size_t kBiasPartFloats = (size_t)kBiasRows * 512;
 
-size_t cnn_grad_floats(int B, int k) {
-    return 2 * (size_t)B * kCh[1] * 64 * 64 + (size_t)B * (kCh[5] + kHidden + 6 * k) + kPartFloats + kBiasPartFloats;
+// the partials' place behind the gradients of the activations, 16-byte aligned
+static size_t part_offset(int B, int k) {
+    return (2 * (size_t)B * kCh[1] * 64 * 64 + (size_t)B * (kCh[5] + kHidden + 6 * k) + 3) & ~(size_t)3;
 }
+
+size_t cnn_grad_floats(int B, int k) { return part_offset(B, k) + kPartFloats + kBiasPartFloats; }
 
 namespace {
 struct Layout {
@@ -781,15 +735,10 @@ cudaError_t launch_cnn_forward(const float *params, int k, const CnnInput &in, i
     k_cnn_stats<<<B, 256, 0, st>>>(in.x, in.img_stride, in.row_stride, in.ox, in.oy, 128, A.affine);
     CNN_TRY(cudaGetLastError());
     int n_launch = 1;
-    int s = 128;
     for (int l = 0; l < 5; ++l) {
-        const int so = s / 2;
-        Src src = l == 0 ? Src{in.x, 1, 128, in.img_stride, in.row_stride, in.ox, in.oy, A.affine}
-                         : Src{A.a[l - 1], kCh[l], s, (long)kCh[l] * s * s, s, 0, 0, nullptr};
-        CNN_TRY(gemm(kCh[l + 1], B * so * so, kCh[l] * 9, 1, LoadW{params + L.cw[l], kCh[l] * 9},
-                     LoadIm2col{src, so}, EpConv{A.a[l], params + L.cb[l], kCh[l + 1], so * so}, st));
+        CNN_TRY(launch_conv32_forward(l, l ? A.a[l - 1] : nullptr, in, A.affine, params + L.cw[l], params + L.cb[l], B,
+                                      A.a[l], st));
         ++n_launch;
-        s = so;
     }
     k_cnn_pool<<<(B * kCh[5] + 255) / 256, 256, 0, st>>>(A.a[4], B * kCh[5], 16, A.pool);
     CNN_TRY(cudaGetLastError());
@@ -859,7 +808,7 @@ cudaError_t launch_cnn_backward(const float *params, int k, const CnnInput &in, 
     const size_t big = (size_t)B * kCh[1] * 64 * 64;
     float *gbufs[2] = {gbuf, gbuf + big};
     float *gout = gbuf + 2 * big, *gh1 = gout + (size_t)B * 6 * k, *gpool = gh1 + (size_t)B * kHidden;
-    float *part = gpool + (size_t)B * kCh[5], *bpart = part + kPartFloats;
+    float *part = gbuf + part_offset(B, k), *bpart = part + kPartFloats;
     int n_launch = 0;
     // weight gradient out[M][N] = A^T B over the batch, reduced over K in splits
     // whose partials are summed in a fixed order (no atomics: reproducible)
@@ -883,7 +832,7 @@ cudaError_t launch_cnn_backward(const float *params, int k, const CnnInput &in, 
         return cudaGetLastError();
     };
     CNN_TRY(cudaMemsetAsync(grad, 0, sizeof(float) * cnn_num_params(k), st));
-    k_cnn_head_loss<<<(B + 127) / 128, 128, 0, st>>>(A.out, B, k, qgt, gout, loss_sum, winners);
+    k_cnn_head_loss<<<(B + kLossWarps - 1) / kLossWarps, 32 * kLossWarps, 0, st>>>(A.out, B, k, qgt, gout, loss_sum, winners);
     CNN_TRY(cudaGetLastError());
     // fc2: dW2 = gout^T h1, db2, gh1 = (W2^T gout) where h1 > 0
     const int M2 = 6 * k;
@@ -898,7 +847,7 @@ cudaError_t launch_cnn_backward(const float *params, int k, const CnnInput &in, 
                  EpStore{gpool, kCh[5]}, st));
     n_launch += 3;
     // mean pool, then the conv layers from the last to the first
-    int so = 4, cur = 0;
+    int cur = 0;
     {
         const long n = (long)B * kCh[5] * 16;
         k_cnn_pool_back<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(gpool, A.a[4], B * kCh[5], 16, gbufs[cur]);
@@ -906,20 +855,15 @@ cudaError_t launch_cnn_backward(const float *params, int k, const CnnInput &in, 
         ++n_launch;
     }
     for (int l = 4; l >= 0; --l) {
-        const int si = 2 * so, ci = kCh[l], co = kCh[l + 1];
         const float *g = gbufs[cur];
-        Src src = l == 0 ? Src{in.x, 1, 128, in.img_stride, in.row_stride, in.ox, in.oy, A.affine}
-                         : Src{A.a[l - 1], ci, si, (long)ci * si * si, si, 0, 0, nullptr};
-        CNN_TRY(weight_grad(co, ci * 9, B * so * so, LoadGradT{g, co, so * so}, LoadIm2colT{src, so},
-                            grad + L.cw[l]));
-        CNN_TRY(bias_grad(g, co, so * so, 2 * num_sms / co, grad + L.cb[l]));
-        if (l > 0) {   // gradient into the previous layer's output, through its ReLU
-            CNN_TRY(gemm(ci, B * si * si, co * 9, 1, LoadWconvT{params + L.cw[l], ci}, LoadGradScatter{g, co, so},
-                         EpMaskedImg{gbufs[cur ^ 1], A.a[l - 1], ci, si * si}, st));
-            ++n_launch;
+        CNN_TRY(launch_conv32_dw(l, g, l ? A.a[l - 1] : nullptr, in, A.affine, B, part, kPartFloats, bpart,
+                                 kBiasPartFloats, grad + L.cw[l], grad + L.cb[l], num_sms, st));
+        n_launch += 3;
+        if (l > 0) {   // gradient into the previous layer's output, through its ReLU (part is free again)
+            CNN_TRY(launch_conv32_dx(l, g, params + L.cw[l], A.a[l - 1], B, part, gbufs[cur ^ 1], st));
+            n_launch += 2;
             cur ^= 1;
         }
-        so = si;
     }
     if (launches) *launches += n_launch;
     return cudaSuccess;

@@ -236,6 +236,20 @@ cudaError_t launch_cnn_forward_bf16(const float *params, int k, const CnnInput &
 // a pipeline wait expired; x, w, y 16-byte aligned
 cudaError_t launch_conv_tc(int layer, const void *x, int B, const void *w, const float *bias, void *y, int *err,
                            int num_sms, cudaStream_t st);
+// FP32 convolution `layer` (0..4), NCHW: y = relu(conv(x) + bias); layer 0 reads
+// the patterns `in` standardised by affine (scale, shift per pattern) instead of
+// x.  Every array 16-byte aligned (not in.x)
+cudaError_t launch_conv32_forward(int layer, const float *x, const CnnInput &in, const float2 *affine, const float *w,
+                                  const float *bias, int B, float *y, cudaStream_t st);
+// its gradient into the input (layers 1..4) through the previous layer's ReLU:
+// gx = conv^T(g) where mask > 0; wt: work array of Co Ci 9 floats
+cudaError_t launch_conv32_dx(int layer, const float *g, const float *w, const float *mask, int B, float *wt, float *gx,
+                             cudaStream_t st);
+// its gradients into the weights (gw [Co][Ci][9]) and the bias (gb [Co]); part
+// and bpart: work arrays of the split sums (at least Co Ci 9 and Co floats)
+cudaError_t launch_conv32_dw(int layer, const float *g, const float *x, const CnnInput &in, const float2 *affine, int B,
+                             float *part, size_t part_floats, float *bpart, size_t bpart_floats, float *gw, float *gb,
+                             int num_sms, cudaStream_t st);
 cudaError_t launch_cnn_forward(const float *params, int k, const CnnInput &in, int B, float *act, int *launches,
                                cudaStream_t st);
 // after launch_cnn_forward on the same act: loss_sum += sum of per-pattern
