@@ -54,7 +54,7 @@ __device__ __forceinline__ void run_item(const MapDev &m, const WorkItem &w, con
         case 96: gen::search_body_reg<96>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g); break;
         case 128:
             if (m.body == kBodyRounds)   // whole CTAs only (phase 0)
-                s128::search_body(m.Stp, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr);
+                s128::search_body<false>(m.Stp, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr);
             else
                 gen::search_body_reg<128>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g);
             break;

@@ -30,10 +30,13 @@
 // carries its selects.  Every shared access of a warp is free of bank
 // conflicts (the swizzles below).
 #include "common.cuh"
+#include "fft128.cuh"
 #include "kernels.cuh"
 #include "project.cuh"
 
 namespace {
+
+using namespace fft128;
 
 constexpr int N = 128, HW = 65, NT = 256, CTAS = 2;
 
@@ -52,20 +55,9 @@ struct Smem {
     float stat[4];               // mean, 1 / deviation, ok | scale, ok
 };
 
-__device__ __forceinline__ float2 w128(int e) {   // e^{+2 pi i e / 128}, 0 <= e < 128
-    const int r = e & 63;
-    const float2 w = make_float2(kTwTable<N>.re[r], kTwTable<N>.im[r]);
-    return e & 64 ? make_float2(-w.x, -w.y) : w;
-}
-
 // image pixel (r, c) as a float of buf: 16-byte pieces swizzled by the row so
 // that eight rows' same columns lie in different banks
 __device__ __forceinline__ int img_at(int r, int c) { return (r << 7) + ((((c >> 2) ^ (r & 7)) << 2) | (c & 3)); }
-// A: (n0 pairs swizzled by pr so that round 2's 16-byte loads of eight
-// consecutive pr fill every bank)
-__device__ __forceinline__ int a_at(int k1, int pr, int n0) {
-    return (k1 << 8) + (pr << 2) + (n0 ^ (((pr >> 2) & 1) << 1));
-}
 // C: one line of 16 y0 per (m, column), its 16-byte pieces swizzled by the column
 __device__ __forceinline__ int c_at(int m, int col, int y0) {
     return (((m << 6) + col) << 4) + ((((y0 >> 1) ^ (col & 7)) << 1) | (y0 & 1));
@@ -80,24 +72,6 @@ __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// 4-point transform of a residue class, SIGN -1 forward
-template <int SIGN>
-__device__ __forceinline__ void dft4(float2 &a, float2 &b, float2 &c, float2 &d) {
-    const float2 s = c_add(a, c), t = c_sub(a, c), u = c_add(b, d);
-    const float2 v = SIGN > 0 ? c_mul_pi(c_sub(b, d)) : c_mul_mi(c_sub(b, d));
-    a = c_add(s, u);
-    b = c_add(t, v);
-    c = c_sub(s, u);
-    d = c_sub(t, v);
-}
-
-// columns of thread (y0, g): g, 32 - g, 32 + g, 64 - g; for g = 0 the packed
-// column (index 0), 16, 32 and 48
-__device__ __forceinline__ int col_of(int g, int k) {
-    return g ? (k == 0 ? g : k == 1 ? 32 - g : k == 2 ? 32 + g : 64 - g)
-             : (k == 0 ? 0 : k == 1 ? 16 : k == 2 ? 32 : 48);
-}
 
 template <Source SRC>
 __global__ void __launch_bounds__(NT, CTAS)
@@ -122,7 +96,8 @@ k_prep128(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
     // round identities
     const int pr = tid >> 2, n0 = tid & 3;                  // 1: row pair, column residue mod 4
     const int y0 = lane & 15, g = 2 * warp + (lane >> 4);   // 2: row residue mod 16, column residue +-g mod 32
-    const int gb = g ? 32 - g : 16;                         //    its second residue
+    const int gb = residue_b(g);                            //    its second residue
+    const bool special = warp == 0 && g == 0;
     const int col = tid & 63, mq = tid >> 6;                // 3: column, u residues mq and mq + 4 mod 8
     // 16-byte copies where every crop row and the output allow them
     const bool vec_in = !PROJ && ((a.W | a.ox) & 3) == 0 && (reinterpret_cast<uintptr_t>(img) & 15) == 0 &&
@@ -229,26 +204,10 @@ k_prep128(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
                 float2 B[4] = {{v0.x, v0.y}, {v0.z, v0.w}, {v1.x, v1.y}, {v1.z, v1.w}};
                 dft4<-1>(A[0], A[1], A[2], A[3]);   // Z at columns g + 32 k
                 dft4<-1>(B[0], B[1], B[2], B[3]);   // Z at columns gb + 32 k
-                // 2 Ra = Z[v] + conj Z[128 - v], 2 Rb = (Z[v] - conj Z[128 - v]) / i (the scale cancels)
-                auto split = [&](float2 zv, float2 zn, float2 &ra, float2 &rb) {
-                    ra = make_float2(zv.x + zn.x, zv.y - zn.y);
-                    rb = make_float2(zv.y + zn.y, zn.x - zv.x);
-                };
-                float2 n1 = A[3], n2 = B[2], n3 = A[2];   // mirrors of columns 32 - g, 32 + g, 64 - g
-                float2 p1 = B[0], p2 = A[1], p3 = B[1];
-                if (warp == 0 && g == 0) {   // columns 16, 32, 48 of the residues 0 and 16
-                    n1 = B[3];
-                    n2 = A[3];
-                    n3 = B[2];
-                }
-                split(p1, n1, x[1][j], x[1][j + 4]);
-                split(p2, n2, x[2][j], x[2][j + 4]);
-                split(p3, n3, x[3][j], x[3][j + 4]);
-                split(A[0], B[3], x[0][j], x[0][j + 4]);
-                if (warp == 0 && g == 0) {   // columns 0 and 64, real: (Ra[0], Ra[64]), (Rb[0], Rb[64])
-                    x[0][j] = make_float2(A[0].x, A[2].x);
-                    x[0][j + 4] = make_float2(A[0].y, A[2].y);
-                }
+                float2 ra[4], rb[4];
+                split_rows(A, B, special, ra, rb);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k][j] = ra[k], x[k][j + 4] = rb[k];
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) fft_reg_dif<8, -1>(x[k]);
@@ -372,17 +331,10 @@ k_prep128(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
                     __syncthreads();   // every thread has read C
                     StaticFor<0, 4>::run([&](auto jj) {
                         constexpr int j = decltype(jj)::value, RA = cx_bitrev(j, 3), RB = cx_bitrev(j + 4, 3);
-                        // Z[v] = Ra + i Rb, Z[128 - v] = conj Ra + i conj Rb
-                        auto zv = [&](int k) { return make_float2(x[k][RA].x - x[k][RB].y, x[k][RA].y + x[k][RB].x); };
-                        auto zn = [&](int k) { return make_float2(x[k][RA].x + x[k][RB].y, x[k][RB].x - x[k][RA].y); };
-                        float2 A[4] = {zv(0), zv(2), zn(3), zn(1)}, B[4] = {zv(1), zv(3), zn(2), zn(0)};
-                        if (warp == 0 && g == 0) {
-                            A[0] = make_float2(x[0][RA].x, x[0][RB].x);
-                            A[2] = make_float2(x[0][RA].y, x[0][RB].y);
-                            A[3] = zn(2);
-                            B[2] = zn(3);
-                            B[3] = zn(1);
-                        }
+                        const float2 ra[4] = {x[0][RA], x[1][RA], x[2][RA], x[3][RA]};
+                        const float2 rb[4] = {x[0][RB], x[1][RB], x[2][RB], x[3][RB]};
+                        float2 A[4], B[4];
+                        merge_rows(ra, rb, special, A, B);
                         dft4<+1>(A[0], A[1], A[2], A[3]);
                         dft4<+1>(B[0], B[1], B[2], B[3]);
                         const int q = y0 + 16 * j;

@@ -5,34 +5,42 @@
 // Discussion (one inverse FFT per pattern-template pair dominates the cost).
 //
 // One CTA (512 threads, one per SM) keeps one pattern's half spectrum in
-// shared memory and streams the library's half spectra from L2/HBM, two
-// templates per inverse FFT: Z = X1 + i X2 with X_j = conj(S_tj) S_p extended
-// to the full spectrum by Hermitian symmetry, so that Re(IFFT Z) and
-// Im(IFFT Z) are the two real correlation surfaces.  The 128 x 128 inverse FFT
-// runs in three register rounds separated by two shared-memory transposes
-// (rows y = k2 + 16 k1 of the column transform, columns x = k3 + 4 k4 of the
-// row transform):
-//   round 1: thread (q, l) owns stored column q and rows u = l + 8m: two
-//            16-point FFTs over m (of X1 and X2), twiddle W128^(l k2); the
-//            conjugate-symmetric partner column 128 - q is written from the
-//            same registers (conj(A1) + i conj(A2) at sub-sequence 8 - l);
-//   round 2: thread (k2, g): radix-8 over l completes the column transform
-//            for rows k2 + 16 k1, then radix-4 over the columns g + 32 i and
-//            twiddle W128^(g k3);
-//   round 3: thread (y, k3): a 32-point FFT over g gives row y, columns
-//            k3 + 4 k4, of both surfaces; the max of each is reduced.
-// Each thread holds 32 complex values per round (at most 128 registers), so
-// sixteen warps share an SM and hide one another's shared-memory latency.
+// shared memory and streams the library's half spectra from L2/HBM.  Its two
+// groups of 256 threads each correlate one template at a time, the even and the
+// odd ones: the real surface of X = conj(S_t) S_p, whose 128 rows are
+// transformed as 64 complex lines (rows y and y + 64 packed, Ra + i Rb), from 64
+// complex columns (columns 0 and 64, real after the column transform, packed in
+// one), 8,192 complex values in 64 KB of shared memory and 32 per thread.  Three
+// register rounds with two shared-memory transposes:
+//   round 1: thread (q, l): stored column q, rows u = l + 8 m: 16-point FFTs
+//            over m for l and l + 4, twiddle W128^(l k2);
+//   round 2: thread (k2, g): radix 8 over l completes rows k2 + 16 j of the
+//            columns +-g mod 32, the rows are paired into lines, radix 4 over
+//            the line's columns g + 32 i, twiddle W128^(g k3);
+//   round 3: thread (line, k3): a 32-point FFT over g gives the columns k3 + 4 k4
+//            of two rows; the maximum is kept per thread.
+// Rounds 2 and 3 of a warp (two k2, all g; eight lines) exchange within the
+// warp: three barriers of the group per template.
+//
+// What bounds it: the FP32 issue of the transforms (15 k warp instructions per
+// template, 12 k of them FP32) and the shared-memory traffic of the exchanges
+// (448 KB) take about the same time, so they have to overlap.  With one
+// template pair per 512-thread CTA (Re and Im the two surfaces of one complex
+// transform) all sixteen warps met at six barriers per pair and did either the
+// one or the other: 168.0 ms for 2,000 patterns x 4,065 templates.  Two groups
+// that share no barrier: 156.0 ms; rounds 2 and 3 within a warp and no exchange
+// for the maximum: 152.8 ms = 33.2 TFLOP/s of algorithmic work, 41 % of the
+// FP32 peak (issue active 65 %, shared-memory pipe 67 %).  Loading the templates
+// straight into registers, without the staging copy, measured 201 ms (no
+// registers left to cover the L2 latency).
 // No surface is written to global memory; only the per-pattern best key (and
 // optionally every per-pair peak) leave the kernel.
 //
 // Library spectra are read in a packed "search layout" (pack_search_layout):
 // for each template, columns 0..63 as [l][m/2][q][m&1] with u = l + 8m (64 KB,
 // so that the 16 rows a round-1 thread needs are 8 conflict-free 16-byte
-// shared loads), then column 64.  The next pair is copied from L2 with
-// cp.async while round 3 computes: round 3 first pulls its values into
-// registers, after which the transpose buffer (128 KB) holds exactly columns
-// 0..63 of two templates.
+// shared loads), then column 64.  A group's next template is copied from L2
+// with cp.async into its buffer while round 3 computes.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -42,6 +50,7 @@ namespace {
 
 using namespace s128;
 
+template <bool ALL>
 __global__ void __launch_bounds__(NT, 1)
 k_search128(const float2 *__restrict__ Spk, int T, const float2 *__restrict__ Sp,
             const int *__restrict__ degen, int pairs_per_cta,
@@ -52,7 +61,7 @@ k_search128(const float2 *__restrict__ Spk, int T, const float2 *__restrict__ Sp
     const int pb = blockIdx.x * pairs_per_cta;
     const int pe = min(npairs, pb + pairs_per_cta);
     if (pb >= pe) return;
-    search_body(Spk, T, Sp, p, pb, pe, keys, peaks_all);
+    search_body<ALL>(Spk, T, Sp, p, pb, pe, keys, peaks_all);
 }
 
 // standard half spectra [T][128][65] -> packed search layout [T][8320]
@@ -79,8 +88,8 @@ cudaError_t launch_pack_search_layout(const float2 *spectra, int T, int N_, floa
 
 cudaError_t launch_search128(const float2 *Spk, int T, const float2 *Sp, const int *degen, int P,
                              unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_search128, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)SMEM_BYTES);
+    auto *kern = peaks_all ? k_search128<true> : k_search128<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const int npairs = (T + 1) / 2;
     // one CTA per SM at a time: split the library into at most max(4, SMs / P)
@@ -101,6 +110,6 @@ cudaError_t launch_search128(const float2 *Spk, int T, const float2 *Sp, const i
     int ppc = (npairs + chunks - 1) / chunks;
     chunks = (npairs + ppc - 1) / ppc;
     dim3 grid(chunks, P);
-    k_search128<<<grid, NT, SMEM_BYTES, st>>>(Spk, T, Sp, degen, ppc, keys, peaks_all);
+    kern<<<grid, NT, SMEM_BYTES, st>>>(Spk, T, Sp, degen, ppc, keys, peaks_all);
     return cudaGetLastError();
 }

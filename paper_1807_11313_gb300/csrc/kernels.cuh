@@ -116,7 +116,7 @@ constexpr int kMapsThreads = 512;   // threads of a queue CTA
 // gives each of the G groups of a CTA maps_smem_bytes() / G, rounded down to
 // 16 bytes, and 512 / G threads)
 inline size_t maps_item_smem(int N, int b, int nt = kMapsThreads) {
-    if (b == kBodyRounds) return (size_t)8 * (128 * 65 + 128 * 128 + 128 + 128 + 256 + 32 + 128);
+    if (b == kBodyRounds) return (size_t)8 * (128 * 65 + 2 * 8192 + 128 + 128 + 512 + 256 + 16);
     if (b == kBodyOct) return (size_t)8 * (64 * 64 + (size_t)(nt / 8) * 72 + 16);
     return (size_t)8 * ((size_t)N * (N + 1) + N + 34);
 }

@@ -1,0 +1,59 @@
+"""All-pairs search at library sizes where its work split ends unevenly (odd
+counts, one template, fewer templates than a part), against float64 inverse
+transforms of the same FP32 spectra.  Bound: 1e-4 relative + 1e-6 on the peaks
+(FP32 transforms of unit-norm spectra), the best template exact."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def px():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1807_11313_gb300 as px
+    px.load()
+    return px
+
+
+def _images(n, P, seed):
+    x = torch.randn((P, n + 4, n + 4), generator=torch.Generator().manual_seed(seed), dtype=torch.float64)
+    x = torch.nn.functional.avg_pool2d(x[:, None], 5, 1)[:, 0]   # correlated pixels, as a pattern's
+    return x.float().cuda().contiguous()
+
+
+def _reference(St, Sp):
+    n = Sp.shape[1]
+    out = torch.stack([torch.fft.irfft2(St.to(torch.complex128).conj() * s.to(torch.complex128), s=(n, n), norm="forward")
+                       .flatten(1).amax(1) for s in Sp])
+    return out
+
+
+def check_search(px, n, T, P, native=0):
+    ctx = px.Context(native_sizes=native)
+    g = px.geometry(n, n)
+    q = torch.zeros((T, 4), dtype=torch.float64, device="cuda")
+    q[:, 0] = 1
+    lib = px.xcf_build_library_images(ctx, _images(n, T, T), q, g)
+    pats = _images(n, P, 1000 + P)
+    if P > 2:
+        pats[1] = 3.0   # degenerate: skipped
+    Sp, _, deg = px.xcf_prep(ctx, pats, g)
+    ref = _reference(lib.spectra(), Sp)
+    ok = deg == 0
+    peaks = px.xcf_correlate_all(ctx, lib, pats)
+    torch.testing.assert_close(peaks[ok].double(), ref[ok], rtol=1e-4, atol=1e-6)
+    assert (peaks[~ok] == 0).all()
+    best, peak, _ = px.xcf_index(ctx, lib, pats)
+    assert (best[~ok] == -1).all()
+    assert torch.equal(best[ok].long(), ref[ok].argmax(1))
+    torch.testing.assert_close(peak[ok].double(), ref[ok].amax(1), rtol=1e-4, atol=1e-6)
+    lib.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 15, 16, 17, 33, 130])
+@pytest.mark.parametrize("P", [1, 3, 153])
+def test_search_128(px, T, P):
+    check_search(px, 128, T, P)
