@@ -1,6 +1,6 @@
 // Pre-processing (N in {16, 32, 64, 96, 160}; 128 in k_prep128.cu), the
-// all-sides search kernel and the single-surface peak kernel for N in {16, 32,
-// 64, 96, 128, 160}.  The search and peak kernels
+// all-sides search kernel for N in {16, 32, 64, 96, 128, 160} and the
+// single-surface peak kernel (128 in k_peak128.cu).  The search and peak kernels
 // hold one N x N complex array in shared memory (rows padded to N + 1) and
 // transform its lines with the warp line FFT (registers and shuffles for
 // N = R x 32 >= 64, mixed radix at 96 and 160; radix-2 butterflies spread
@@ -43,7 +43,7 @@ constexpr size_t smem_prep_real() {
 // threads per CTA: more warps for the larger sides hide the shared-memory and
 // global-load latency of the line transforms
 template <int N>
-constexpr int peak_threads() { return N >= 128 ? 1024 : kThreads; }
+constexpr int peak_threads() { return N > 128 ? 1024 : kThreads; }
 template <int N>
 __host__ __device__ constexpr int search_threads() { return N >= 128 ? 1024 : kThreads; }
 
@@ -739,7 +739,7 @@ cudaError_t launch_pair_peak(int N, const float2 *St, const int *tidx, const flo
         case 16: return pair_peak_n<16>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
         case 32: return pair_peak_n<32>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
         case 64: return pair_peak_n<64>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
-        case 128: return pair_peak_n<128>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
+        case 128: return launch_peak128(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
         case 96: return pair_peak_n<96>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
         case 160: return pair_peak_n<160>(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);
         case 200: return launch_pair_peak_n200(St, tidx, Sp, degen, active, P, peak, shift, argmax, st);

@@ -135,6 +135,9 @@ cudaError_t launch_pack_search_layout(const float2 *spectra, int T, int N, float
 cudaError_t launch_pair_peak(int N, const float2 *St, const int *tidx, const float2 *Sp,
                              const int *degen, const int *active, int P, float *peak, float *shift,
                              cudaStream_t st, int *argmax = nullptr);
+// the same for N = 128 (k_peak128.cu)
+cudaError_t launch_peak128(const float2 *St, const int *tidx, const float2 *Sp, const int *degen, const int *active,
+                           int P, float *peak, float *shift, int *argmax, cudaStream_t st);
 // up-sampled peak (U >= 2): the correlation's Fourier series on a +-1 px grid of step 1/U
 // around argmax[p]; overwrites peak and shift of every computed pattern
 cudaError_t launch_upsample_peak(int N, const float2 *St, const int *tidx, const float2 *Sp, const int *degen,

@@ -57,3 +57,36 @@ def check_search(px, n, T, P, native=0):
 @pytest.mark.parametrize("P", [1, 3, 153])
 def test_search_128(px, T, P):
     check_search(px, 128, T, P)
+
+
+@pytest.mark.parametrize("dy", [0, 1, 63, 64, 65, 127])
+@pytest.mark.parametrize("dx", [0, 1, 63, 64, 127])
+def test_peak_128_at_every_wrap(px, dy, dx):
+    """A circularly shifted, unwindowed pattern peaks at exactly that shift,
+    wrapped into [-64, 64); the parabola of a symmetric peak adds nothing
+    (1e-3 px: FP32 differences of neighbouring values near 1)."""
+    n = 128
+    ctx = px.Context(window=0)
+    g = px.geometry(n, n)
+    img = _images(n, 1, 7)
+    q = torch.tensor([[1.0, 0, 0, 0]], dtype=torch.float64, device="cuda")
+    lib = px.xcf_build_library_images(ctx, img, q, g)
+    best, peak, shift = px.xcf_index(ctx, lib, torch.roll(img, (dy, dx), (1, 2)).contiguous())
+    want = [float(d if d < n // 2 else d - n) for d in (dx, dy)]
+    assert best.tolist() == [0] and abs(peak.item() - 1) < 1e-5
+    torch.testing.assert_close(shift[0].cpu(), torch.tensor(want), rtol=0, atol=1e-3)
+    lib.close()
+    ctx.close()
+
+
+def test_peak_128_tie_takes_the_lowest_shift(px):
+    """A template without signal gives a surface of equal values: index 0."""
+    n = 128
+    ctx = px.Context()
+    g = px.geometry(n, n)
+    q = torch.tensor([[1.0, 0, 0, 0]], dtype=torch.float64, device="cuda")
+    lib = px.xcf_build_library_images(ctx, torch.full((1, n, n), 2.0, device="cuda"), q, g)
+    best, peak, shift = px.xcf_index(ctx, lib, _images(n, 3, 9))
+    assert best.tolist() == [0] * 3 and peak.tolist() == [0] * 3 and (shift == 0).all()
+    lib.close()
+    ctx.close()
