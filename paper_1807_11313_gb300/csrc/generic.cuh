@@ -101,23 +101,59 @@ __device__ void make_twiddles(float2 *tw, int sign) {
     make_twiddles<N>(tw, sign, (int)threadIdx.x, (int)blockDim.x);
 }
 
-// sum over the block of one FP32 partial per thread: warp sums in FP32, the
-// warps' sums added in FP64 (keeps the hot loops off the FP64 pipe)
-__device__ inline double block_sum_f(float v, double *sh) {
+// Statistics of a crop from one FP32 partial per thread of the sums of d = x - x0
+// and d^2 over n pixels, and the scale of its filtered spectrum from one partial
+// of the energy: warp sums in FP32, the warps' sums and everything after them in
+// FP64, by thread 0 alone.  (GB300's FP64 pipe is narrow: evaluated by every
+// thread, the square roots and divisions took a third to a half of an image's
+// pre-processing.)
+struct CropStats {
+    float mean, inv;   // mean and 1 / standard deviation of the crop
+    bool bad;          // no variance
+};
+__device__ inline CropStats block_stats(float s1, float s2, float x0, int n) {
+    __shared__ float2 part[32];
+    __shared__ float2 res;
+    __shared__ int res_bad;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[w] = (double)v;
+    for (int o = 16; o; o >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+    if (lane == 0) part[w] = make_float2(s1, s2);
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nw; ++i) s += sh[i];
-        sh[32] = s;
+        double t1 = 0.0, t2 = 0.0;
+        for (int i = 0; i < nw; ++i) {
+            t1 += (double)part[i].x;
+            t2 += (double)part[i].y;
+        }
+        const double m1 = t1 / n, mean = x0 + m1, var = t2 / n - m1 * m1;
+        const double sd = var > 0.0 ? sqrt(var) : 0.0;
+        const bool bad = !(sd > 1e-12 * (1.0 + fabs(mean)));
+        res = make_float2((float)mean, bad ? 0.f : (float)(1.0 / sd));
+        res_bad = bad;
     }
     __syncthreads();
-    const double r = sh[32];
+    return CropStats{res.x, res.y, res_bad != 0};
+}
+// 1 / sqrt(energy), 0 where there is none
+__device__ inline float block_scale(float e) {
+    __shared__ float part[32];
+    __shared__ float res;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) part[w] = e;
     __syncthreads();
-    return r;
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int i = 0; i < nw; ++i) t += (double)part[i];
+        res = t > 0.0 ? (float)(1.0 / sqrt(t)) : 0.f;
+    }
+    __syncthreads();
+    return res;
 }
 
 // max over the unit of one value per thread (sh: 33 floats of the unit's own)

@@ -705,20 +705,21 @@ __device__ __forceinline__ double ld_cluster_d(uint32_t addr) {
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
     return v;
 }
-// FP32 partial per thread: warp sums in FP32, the warps' sums in FP64
-__device__ __forceinline__ double block_sum_fd(float v, double *sh) {
+// FP32 partials per thread: warp sums in FP32, the warps' sums in FP64, by thread
+// 0 alone (GB300's FP64 pipe is narrow: with every thread evaluating the sums,
+// square roots and divisions they took a third of an image's time)
+__device__ __forceinline__ double block_sum_fd(float v, double *sh) {   // in thread 0
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = (double)v;
     __syncthreads();
     double s = 0.0;
-    for (int w = 0; w < NT / 32; ++w) s += sh[w];
+    if (threadIdx.x == 0)
+        for (int w = 0; w < NT / 32; ++w) s += sh[w];
     __syncthreads();
     return s;
 }
-// sum of one partial per CTA, identical (same order) in every CTA of the cluster
-__device__ __forceinline__ double cluster_sum(double part, double *slot, uint32_t slot_addr) {
-    if (threadIdx.x == 0) *slot = part;
-    cluster_barrier();
+// sum of the slots of the cluster's CTAs, in the same order in every CTA
+__device__ __forceinline__ double slot_sum(uint32_t slot_addr) {
     double s = 0.0;
     for (int r = 0; r < NC; ++r) s += ld_cluster_d(map_to_rank(slot_addr, r));
     return s;
@@ -736,6 +737,7 @@ k_prep_c256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict
     float2 *scr_all = Col128 + N;
     double *red = reinterpret_cast<double *>(scr_all + SCR_F2);   // [0..7] block partials, [8..10] cluster slots
     float *Xr = reinterpret_cast<float *>(red + 16);              // this CTA's 64 input rows [64][256]
+    __shared__ float stat[4];                                     // mean, 1 / deviation, none | scale
     const int tid = threadIdx.x, t = tid & 15, g = tid >> 4;
     const int c = (int)cluster_rank();
     const int cid = blockIdx.x / NC, ncl = gridDim.x / NC;
@@ -800,17 +802,25 @@ k_prep_c256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict
         }
         const double s = block_sum_fd(sf, red);
         const double s2 = block_sum_fd(sf2, red);
-        if (tid == 0) red[9] = s2;
-        const double tot = cluster_sum(s, red + 8, slot_local);   // its barrier also publishes red[9]
-        double tot2 = 0.0;
-        for (int r = 0; r < NC; ++r) tot2 += ld_cluster_d(map_to_rank(slot_local + sizeof(double), r));
-        const double m1 = tot / ((double)N * N);
-        const double mean = x0 + m1;
-        const double sd = sqrt(fmax(tot2 / ((double)N * N) - m1 * m1, 0.0));
-        bool bad = !(sd > 1e-12 * (1.0 + fabs(mean)));
+        if (tid == 0) {
+            red[8] = s;
+            red[9] = s2;
+        }
+        cluster_barrier();   // publishes the slots
+        if (tid == 0) {
+            const double m1 = slot_sum(slot_local) / ((double)N * N);
+            const double mean = x0 + m1;
+            const double sd = sqrt(fmax(slot_sum(slot_local + sizeof(double)) / ((double)N * N) - m1 * m1, 0.0));
+            const bool none = !(sd > 1e-12 * (1.0 + fabs(mean)));
+            stat[0] = (float)mean;
+            stat[1] = none ? 0.f : (float)(1.0 / sd);
+            stat[2] = none ? 1.f : 0.f;
+        }
+        __syncthreads();
+        bool bad = stat[2] != 0.f;
         if (!bad) {
             // ---- rows (two per complex line), windowed and standardised
-            const float m = (float)mean, inv = (float)(1.0 / sd);
+            const float m = stat[0], inv = stat[1];
 #pragma unroll 1
             for (int q = 0; q < 2; ++q) {
                 const int ra = 2 * (g + 16 * q), rb = ra + 1;
@@ -879,8 +889,16 @@ k_prep_c256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict
                 }
             }
         }
-        const double energy = cluster_sum(block_sum_fd(e, red), red + 10, slot_local + 2 * sizeof(double));
-        bad = bad || !(energy > 0.0);
+        const double part = block_sum_fd(e, red);
+        if (tid == 0) red[10] = part;
+        cluster_barrier();
+        if (tid == 0) {
+            const double energy = slot_sum(slot_local + 2 * sizeof(double));
+            stat[3] = energy > 0.0 ? (float)(1.0 / sqrt(energy)) : 0.f;
+        }
+        __syncthreads();
+        const float sc = stat[3];
+        bad = bad || !(sc > 0.f);
         if (tid == 0 && c == 0 && degen) degen[p] = bad ? 1 : 0;
         if (bad) {
             for (int i = tid; i < ROWS * HW; i += NT) out[(size_t)ROWS * c * HW + i] = make_float2(0.f, 0.f);
@@ -888,7 +906,6 @@ k_prep_c256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict
                 for (int i = tid; i < ROWS * N; i += NT) spatial[(size_t)p * N * N + (size_t)ROWS * c * N + i] = 0.f;
             continue;   // uniform: the decision used cluster-wide sums
         }
-        const float sc = (float)(1.0 / sqrt(energy));
         for (int i = tid; i < N * 32; i += NT) {
             const int u = i >> 5, vl = i & 31;
             const float2 X = Stage[st_index(u, vl)];

@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
     float2 *twHi = twH + N / 4;
     float2 *c0 = twHi + N / 4;                             // S[u][0],   u < N
     float2 *cH = c0 + N;                                   // S[u][N/2], u < N
-    __shared__ double red[33];
     // per-index tables: the Hann window, and the band-pass as a product of
     // per-frequency factors (e(f) = expm1(-f^2 / 2 s_h^2), b(f) = exp(-f^2 / 2 s_l^2):
     // 1 - exp(-(x_u + x_v)) = -(e_u + e_v + e_u e_v), free of cancellation near DC)
@@ -117,13 +116,11 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
             take(r, c, pixel(r, c));
         }
     }
-    const double m1 = block_sum_f(s1, red) / (N * N), m2 = block_sum_f(s2, red) / (N * N);
-    const double mean = x0 + m1, var = m2 - m1 * m1;
-    const double sd = var > 0.0 ? sqrt(var) : 0.0;
-    bool bad = !(sd > 1e-12 * (1.0 + fabs(mean)));
-    double energy = 0.0;
+    const CropStats cs = block_stats(s1, s2, x0, N * N);
+    bool bad = cs.bad;
+    float sc = 0.f;
     if (!bad) {
-        const float m = (float)mean, inv = (float)(1.0 / sd);
+        const float m = cs.mean, inv = cs.inv;
         for (int idx = tid; idx < H * N; idx += PT) {
             const int pr = idx / N, c = idx % N;
             const float wc = win[c] * inv, w0 = win[2 * pr], w1 = win[2 * pr + 1];
@@ -203,8 +200,8 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
             *x = X;
             e = fmaf(v == 0 || v == N / 2 ? 1.f : 2.f, X.x * X.x + X.y * X.y, e);
         }
-        energy = block_sum_f(e, red);
-        bad = !(energy > 0.0);
+        sc = block_scale(e);
+        bad = !(sc > 0.f);
     }
     if (tid == 0 && degen) degen[p] = bad ? 1 : 0;
     if (bad) {
@@ -213,7 +210,6 @@ __global__ void __launch_bounds__(PT) k_prep_real(const float *__restrict__ img,
             for (int idx = tid; idx < N * N; idx += PT) spatial[(size_t)p * N * N + idx] = 0.f;
         return;
     }
-    const float sc = (float)(1.0 / sqrt(energy));
     for (int it = tid; it < N * HW; it += PT) {
         const int u = it / HW, v = it % HW;
         const float2 X = v == 0 ? c0[u] : (v == N / 2 ? cH[u] : buf[(u & (H - 1)) * LD + (u >= H ? N / 2 : 0) + v]);
@@ -312,7 +308,6 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
     float2 *buf = reinterpret_cast<float2 *>(smem_raw);
     float2 *twf = buf + N * LD, *twi = twf + N / 2;
     float2 *cA0 = twi + N / 2, *cAH = cA0 + N, *cB0 = cAH + N, *cBH = cB0 + N;
-    __shared__ double red[33];
     const int tid = threadIdx.x;
     const int pa = 2 * blockIdx.x, pb = pa + 1;
     const bool ha = pa < P && (!active || active[pa]);
@@ -336,16 +331,12 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
         b1 += db;
         b2 = fmaf(db, db, b2);
     }
-    const double A1 = block_sum_f(a1, red) / (N * N), A2 = block_sum_f(a2, red) / (N * N);
-    const double B1 = block_sum_f(b1, red) / (N * N), B2 = block_sum_f(b2, red) / (N * N);
-    const double meanA = xa0 + A1, varA = A2 - A1 * A1, sdA = varA > 0.0 ? sqrt(varA) : 0.0;
-    const double meanB = xb0 + B1, varB = B2 - B1 * B1, sdB = varB > 0.0 ? sqrt(varB) : 0.0;
-    bool badA = !ha || !(sdA > 1e-12 * (1.0 + fabs(meanA)));
-    bool badB = !hb || !(sdB > 1e-12 * (1.0 + fabs(meanB)));
+    const CropStats csA = block_stats(a1, a2, xa0, N * N), csB = block_stats(b1, b2, xb0, N * N);
+    bool badA = !ha || csA.bad, badB = !hb || csB.bad;
     // ---- standardise and window (a degenerate crop becomes zeros)
     {
-        const float mA = (float)meanA, iA = badA ? 0.f : (float)(1.0 / sdA);
-        const float mB = (float)meanB, iB = badB ? 0.f : (float)(1.0 / sdB);
+        const float mA = csA.mean, iA = badA ? 0.f : csA.inv;
+        const float mB = csB.mean, iB = badB ? 0.f : csB.inv;
         for (int idx = tid; idx < N * N; idx += NT) {
             const int r = idx / N, c = idx - r * N;
             const float w = a.window ? 0.25f * (1.f - cospif(2.f * r / N)) * (1.f - cospif(2.f * c / N)) : 1.f;
@@ -387,14 +378,15 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
         (v ? cAH : cA0)[u] = XA;
         (v ? cBH : cB0)[u] = XB;
     }
-    const double EA = block_sum_f(eA, red), EB = block_sum_f(eB, red);   // its barriers order the writes above
-    badA = badA || !(EA > 0.0);
-    badB = badB || !(EB > 0.0);
+    float sA = block_scale(eA), sB = block_scale(eB);   // their barriers order the writes above
+    badA = badA || !(sA > 0.f);
+    badB = badB || !(sB > 0.f);
+    if (badA) sA = 0.f;
+    if (badB) sB = 0.f;
     if (tid == 0 && degen) {
         if (ha) degen[pa] = badA ? 1 : 0;
         if (hb) degen[pb] = badB ? 1 : 0;
     }
-    const float sA = badA ? 0.f : (float)(1.0 / sqrt(EA)), sB = badB ? 0.f : (float)(1.0 / sqrt(EB));
     float2 *oa = spec + (size_t)pa * N * HW, *ob = spec + (size_t)pb * N * HW;
     for (int it = tid; it < N * HW; it += NT) {
         const int u = it / HW, v = it - u * HW;

@@ -147,22 +147,28 @@ __global__ void __launch_bounds__(256) k_logpolar_img(const float *__restrict__ 
     }
 }
 
-// FP32 partial per thread: warp sums in FP32, the warps' sums in FP64
-__device__ double block_sum_fd(float v, double *sh) {
+// means of two FP32 partials per thread over n values: warp sums in FP32, the
+// warps' sums and the division in FP64 by thread 0 alone (GB300's FP64 pipe is
+// narrow); sh: one entry per warp, and one for the result
+__device__ float2 block_means(float a, float b, int n, float2 *sh) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[w] = (double)v;
+    for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) sh[w] = make_float2(a, b);
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < nw; ++k) s += sh[k];
-        sh[32] = s;
+        double s = 0.0, t = 0.0;
+        for (int k = 0; k < nw; ++k) {
+            s += (double)sh[k].x;
+            t += (double)sh[k].y;
+        }
+        sh[nw] = make_float2((float)(s / n), (float)(t / n));
     }
     __syncthreads();
-    const double r = sh[32];
-    __syncthreads();
-    return r;
+    return sh[nw];
 }
 
 __device__ __forceinline__ float parabola(float cm, float c0, float cp) {
@@ -198,7 +204,7 @@ __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update
     __shared__ float2 tw[NETA / 2], twi[NETA / 2];
     __shared__ float2 zc[NETA];
     __shared__ float cfin[NETA];
-    __shared__ double red[33];
+    __shared__ float2 red[kEtaWarps + 1];
     __shared__ double wshift[kMaxLpWindows];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const float *ga = lpT + (size_t)p * nr * NETA, *gb = lpP + (size_t)p * nr * NETA;
@@ -215,8 +221,8 @@ __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update
         const int i0 = m0 * NETA, i1 = m1 * NETA;
         float s1 = 0.f, s2 = 0.f;
         for (int i = i0 + tid; i < i1; i += kEtaThreads) { s1 += ga[i]; s2 += gb[i]; }
-        const float ma = (float)(block_sum_fd(s1, red) / (i1 - i0));
-        const float mb = (float)(block_sum_fd(s2, red) / (i1 - i0));
+        const float2 mean = block_means(s1, s2, i1 - i0, red);
+        const float ma = mean.x, mb = mean.y;
         float2 acc[KPL];
 #pragma unroll
         for (int j = 0; j < KPL; ++j) acc[j] = make_float2(0.f, 0.f);

@@ -182,7 +182,6 @@ __global__ void __launch_bounds__(NT, 1) k_prep_n200(const float *__restrict__ i
     extern __shared__ float4 smem_raw[];
     float2 *buf = reinterpret_cast<float2 *>(smem_raw);
     float2 *tw = buf + OFF_TW;
-    __shared__ double red[33];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float2 *sa = buf + OFF_SCR + warp * 2 * N, *sb = sa + N;
     make_tw200(tw);
@@ -197,13 +196,11 @@ __global__ void __launch_bounds__(NT, 1) k_prep_n200(const float *__restrict__ i
         s1 += d;
         s2 = fmaf(d, d, s2);
     }
-    const double m1 = gen::block_sum_f(s1, red) / (N * N), m2 = gen::block_sum_f(s2, red) / (N * N);
-    const double mean = x0 + m1, var = m2 - m1 * m1;
-    const double sd = var > 0.0 ? sqrt(var) : 0.0;
-    bool bad = !(sd > 1e-12 * (1.0 + fabs(mean)));
-    double energy = 0.0;
+    const gen::CropStats cs = gen::block_stats(s1, s2, x0, N * N);
+    bool bad = cs.bad;
+    float sc = 0.f;
     if (!bad) {
-        const float mf = (float)mean, inv = (float)(1.0 / sd);
+        const float mf = cs.mean, inv = cs.inv;
         // rows: the standardised, windowed row as 100 complex points (x[2n], x[2n + 1]),
         // transformed, then split into its half spectrum X[k] = E[k] + e^{-2 pi i k / 200} O[k]
         for (int y = warp; y < N; y += NWARP) {
@@ -238,8 +235,8 @@ __global__ void __launch_bounds__(NT, 1) k_prep_n200(const float *__restrict__ i
             buf[it] = X;
             e = fmaf(v == 0 || v == N / 2 ? 1.f : 2.f, X.x * X.x + X.y * X.y, e);
         }
-        energy = gen::block_sum_f(e, red);
-        bad = !(energy > 0.0);
+        sc = gen::block_scale(e);
+        bad = !(sc > 0.f);
     }
     if (tid == 0 && degen) degen[p] = bad ? 1 : 0;
     if (bad) {
@@ -248,7 +245,6 @@ __global__ void __launch_bounds__(NT, 1) k_prep_n200(const float *__restrict__ i
             for (int idx = tid; idx < N * N; idx += NT) spatial[(size_t)p * N * N + idx] = 0.f;
         return;
     }
-    const float sc = (float)(1.0 / sqrt(energy));
     for (int it = tid; it < N * HW; it += NT) out[it] = make_float2(buf[it].x * sc, buf[it].y * sc);
     if (!spatial) return;
     // ---- filtered image: the unit-norm spectrum back through the columns and the rows, / N

@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kNormThreads = 256, kRescoreThreads = 256;
 
+// the block's sum, in thread 0
 __device__ __forceinline__ double block_sum_d(double v, double *red) {
     const int tid = threadIdx.x, nw = blockDim.x >> 5;
 #pragma unroll
@@ -33,7 +34,8 @@ __device__ __forceinline__ double block_sum_d(double v, double *red) {
     if ((tid & 31) == 0) red[tid >> 5] = v;
     __syncthreads();
     double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += red[w];
+    if (tid == 0)   // the only user (GB300's FP64 pipe is narrow)
+        for (int w = 0; w < nw; ++w) s += red[w];
     return s;
 }
 
@@ -55,11 +57,20 @@ __global__ void __launch_bounds__(kNormThreads) k_ndp_norm(const float *__restri
         s2 = fmaf(v, v, s2);
     }
     const double S1 = block_sum_d(s1, red), S2 = block_sum_d(s2, red);
-    const double m1 = S1 / d, var = S2 / d - m1 * m1;
-    const double mean = x0 + m1, sd = var > 0.0 ? sqrt(var) : 0.0;
-    const bool bad = !(sd > 1e-12 * (1.0 + fabs(mean)));
-    if (tid == 0 && degen) degen[p] = bad ? 1 : 0;
-    const float m = (float)mean, scale = bad ? 0.f : (float)(1.0 / (sd * n));
+    __shared__ float res[2];
+    __shared__ int res_bad;
+    if (tid == 0) {
+        const double m1 = S1 / d, var = S2 / d - m1 * m1;
+        const double mean = x0 + m1, sd = var > 0.0 ? sqrt(var) : 0.0;
+        const bool none = !(sd > 1e-12 * (1.0 + fabs(mean)));
+        res[0] = (float)mean;
+        res[1] = none ? 0.f : (float)(1.0 / (sd * n));
+        res_bad = none;
+        if (degen) degen[p] = none ? 1 : 0;
+    }
+    __syncthreads();
+    const bool bad = res_bad != 0;
+    const float m = res[0], scale = res[1];
     float *o32 = out32 ? out32 + (size_t)p * d : nullptr;
     __nv_bfloat16 *o16 = out16 ? out16 + (size_t)p * d : nullptr;
     for (long i = tid; i < d; i += kNormThreads) {
