@@ -372,10 +372,9 @@ int xcf_nearest_disorientation(xcf_ctx *ctx, const double *qa, int32_t na, const
  *                    shared-memory transposes (the kernel of xcf_index);
  *   XCF_BODY_SMEM    N = 16, 32, 64: the surface in shared memory, radix-2
  *                    line transforms;
- *   XCF_BODY_OCT     N = 64 only: eight-lane groups, a 64-point line as an
- *                    8-point FFT in registers, a twiddle, a shared-memory
- *                    transpose and a second 8-point FFT (the kernel of
- *                    xcf_index at N = 64);
+ *   XCF_BODY_OCT     N = 64 only: three register rounds (8-point column FFTs;
+ *                    radix 8 x 2; 32-point row FFTs) of one template on a unit
+ *                    of 64 threads (the kernel of xcf_index at N = 64);
  * the number of patterns a CTA searches side by side (1, 2 or 4 groups of
  * warps, each with its share of the shared memory, where the body fits), and
  * the granularity, the number of template pairs per work item (the whole

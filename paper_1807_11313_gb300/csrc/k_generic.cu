@@ -12,8 +12,8 @@
 #include "common.cuh"
 #include "generic.cuh"
 #include "kernels.cuh"
-#include "oct64.cuh"
 #include "project.cuh"
+#include "rounds.cuh"
 
 namespace {
 
@@ -441,20 +441,24 @@ __global__ void __launch_bounds__(search_threads<N>()) k_search_generic(const fl
     search_body<N, (search_threads<N>() <= 512)>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
 }
 
-// N = 64: the eight-lane-group body (8 x 8 line transforms) on 128-thread
-// CTAs, several resident per SM
-constexpr int kOctThreads = 128;
-__global__ void __launch_bounds__(kOctThreads) k_search_oct64(const float2 *__restrict__ St, int T,
-                                                             const float2 *__restrict__ Sp,
-                                                             const int *__restrict__ degen, int pairs_per_cta,
-                                                             unsigned long long *__restrict__ keys,
-                                                             float *__restrict__ peaks_all,
-                                                             const int *__restrict__ cand, int kc) {
+// N = 64 and 96: three register rounds on units of 64 and 192 threads: at 64 two
+// units per CTA and four CTAs per SM, at 96 four units in one CTA per SM (two
+// CTAs of two, which need the pattern twice, spill more: 20.9 against 27.5
+// TFLOP/s; three units without spills 26.7).  2,000 patterns x 2,000 templates at
+// 64: 27.3 -> 16.3 ms (19.9 -> 33.2 TFLOP/s) against eight-lane line transforms,
+// 1,000 x 2,000 at 96: 41.9 -> 24.1 ms (15.8 -> 27.5) against warp-line transforms.
+template <int N>
+constexpr int rounds_threads() { return (N == 64 ? 2 : 4) * rnd::Shape<N>::UT; }
+template <int N, bool ALL>
+__global__ void __launch_bounds__(rounds_threads<N>(), N == 64 ? 4 : 1)
+k_search_rounds(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, const int *__restrict__ degen,
+                int pairs_per_cta, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
+                const int *__restrict__ cand, int kc) {
     const int p = blockIdx.y;
     if (degen[p]) return;
     const int npairs = ((cand ? kc : T) + 1) / 2;
     const int pb = blockIdx.x * pairs_per_cta, pe = min(npairs, pb + pairs_per_cta);
-    o64::search_body(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc, gen::cta_group());
+    rnd::search_body<N, ALL>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc, gen::cta_group());
 }
 
 __device__ __forceinline__ float parabola(float cm, float c0, float cp) {
@@ -614,18 +618,20 @@ cudaError_t search_n(const float2 *St, int T, const float2 *Sp, const int *degen
                      unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st,
                      const int *cand = nullptr, int kc = 0) {
     const int npairs = ((cand ? kc : T) + 1) / 2;
-    if constexpr (N == 64) {   // 128-thread CTAs: enough to fill every SM four deep a few times over
-        const size_t sm = o64::smem_bytes(kOctThreads);
-        cudaError_t e = set_smem(k_search_oct64, sm);
+    if constexpr (N == 64 || N == 96) {   // enough CTAs to fill every SM a few times over, at least 4 pairs each
+        constexpr int NT = rounds_threads<N>();
+        const size_t sm = rnd::smem_bytes<N>(NT);
+        auto *kern = peaks_all ? k_search_rounds<N, true> : k_search_rounds<N, false>;
+        cudaError_t e = set_smem(kern, sm);
         if (e != cudaSuccess) return e;
         const long want = (long)num_sms * 32;
         int chunks = (int)((want + P - 1) / P);
         chunks = max(1, min(chunks, (npairs + 3) / 4));
         int ppc = (npairs + chunks - 1) / chunks;
         chunks = (npairs + ppc - 1) / ppc;
-        k_search_oct64<<<dim3(chunks, P), kOctThreads, sm, st>>>(St, T, Sp, degen, ppc, keys, peaks_all, cand, kc);
+        kern<<<dim3(chunks, P), NT, sm, st>>>(St, T, Sp, degen, ppc, keys, peaks_all, cand, kc);
         return cudaGetLastError();
-    }
+    } else {
     size_t sm = gen::smem_bytes<N>();
     cudaError_t e = set_smem(k_search_generic<N>, sm);
     if (e != cudaSuccess) return e;
@@ -638,6 +644,7 @@ cudaError_t search_n(const float2 *St, int T, const float2 *Sp, const int *degen
     dim3 grid(chunks, P);
     k_search_generic<N><<<grid, search_threads<N>(), sm, st>>>(St, T, Sp, degen, ppc, keys, peaks_all, cand, kc);
     return cudaGetLastError();
+    }
 }
 
 template <int N>

@@ -88,7 +88,7 @@ cudaError_t launch_to_bf16(const float *x, size_t n, void *y, cudaStream_t st);
 constexpr int kBodyReg = 0;      // register warp-line transforms (N = R x 32: 64, 96, 128, 160)
 constexpr int kBodyRounds = 1;   // N = 128: three register rounds with two shared-memory transposes
 constexpr int kBodySmem = 2;     // surface in shared memory, radix-2 line transforms (2^k sides up to 64)
-constexpr int kBodyOct = 3;      // N = 64: eight-lane groups, 8 x 8 line transforms with shared-memory transposes
+constexpr int kBodyOct = 3;      // N = 64: three register rounds on units of 64 threads
 constexpr int kNumBodies = 4;
 struct MapDev {
     int N, T, body;                // detector side, library size, search body (items of the map run on
@@ -117,7 +117,7 @@ constexpr int kMapsThreads = 512;   // threads of a queue CTA
 // 16 bytes, and 512 / G threads)
 inline size_t maps_item_smem(int N, int b, int nt = kMapsThreads) {
     if (b == kBodyRounds) return (size_t)8 * (128 * 65 + 2 * 8192 + 128 + 128 + 512 + 256 + 16);
-    if (b == kBodyOct) return (size_t)8 * (64 * 64 + (size_t)(nt / 8) * 72 + 16);
+    if (b == kBodyOct) return (size_t)8 * (64 * 33 + 128 + (size_t)(nt / 64) * (32 * 64 + 64));
     return (size_t)8 * ((size_t)N * (N + 1) + N + 34);
 }
 // Items are ordered by phase: [offs[0], offs[1]) run on whole CTAs, [offs[1],

@@ -90,3 +90,42 @@ def test_peak_128_tie_takes_the_lowest_shift(px):
     assert best.tolist() == [0] * 3 and peak.tolist() == [0] * 3 and (shift == 0).all()
     lib.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 7, 8, 9, 33, 130])
+@pytest.mark.parametrize("P", [1, 3, 40])
+@pytest.mark.parametrize("n", [64, 96])
+def test_search_64_and_96(px, n, T, P):
+    check_search(px, n, T, P, native=1)
+
+
+@pytest.mark.parametrize("n", [64, 96])
+@pytest.mark.parametrize("k", [1, 2, 5, 8])
+def test_candidate_lists_64_and_96(px, n, k):
+    """Lists with empty entries, repeated templates (ties to the lowest index)
+    and descending order against float64."""
+    T, P = 20, 5
+    ctx = px.Context(native_sizes=1)
+    g = px.geometry(n, n)
+    q = torch.zeros((T, 4), dtype=torch.float64, device="cuda")
+    q[:, 0] = 1
+    imgs = _images(n, T, 5)
+    imgs[11] = imgs[4]
+    lib = px.xcf_build_library_images(ctx, imgs, q, g)
+    pats = torch.cat([imgs[11:12], _images(n, P - 1, 6)])
+    cand = torch.tensor([[11, 4, -1, 19, 0, 7, -1, 3], [-1] * 8, [0, 1, 2, 3, 4, 5, 6, 7], [19, 18, 17, 16, 15, 14, 13, 12],
+                         [4, -1, 11, -1, 4, 9, 9, 9]], dtype=torch.int32, device="cuda")[:, :k].contiguous()
+    best, peak, _ = px.xcf_rescore(ctx, lib, pats, cand)
+    ref = _reference(lib.spectra(), px.xcf_prep(ctx, pats, g)[0])
+    for p in range(P):
+        c = sorted({int(t) for t in cand[p] if t >= 0})
+        if not c:
+            assert best[p] == -1 and peak[p] == 0
+            continue
+        top = max(c, key=lambda t: (ref[p, t].item(), -t))
+        if ref[p, top] - ref[p, 4] < 1e-7 and 4 in c:   # equal templates 4 and 11
+            top = 4
+        assert int(best[p]) == top
+        torch.testing.assert_close(peak[p].double(), ref[p, top], rtol=1e-4, atol=1e-6)
+    lib.close()
+    ctx.close()
