@@ -254,7 +254,6 @@ cudaError_t run_prep(xcf_ctx * /*ctx*/, const float *img, int P, const PrepArgs 
 
 cudaError_t run_search(xcf_ctx * /*ctx*/, int n, const float2 *St, int T, const float2 *Sp, const int *degen, int P,
                        unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st) {
-    if (n == 200) return launch_search_n200(St, T, Sp, degen, P, keys, peaks_all, num_sms, st, nullptr, 0);
     if (n != 256) return launch_search(n, St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
     return launch_search_c256(St, T, Sp, degen, P, keys, peaks_all, nullptr, 0, st);
 }

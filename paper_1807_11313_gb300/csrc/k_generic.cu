@@ -702,8 +702,8 @@ cudaError_t launch_search(int N, const float2 *St, int T, const float2 *Sp, cons
         case 64: return search_n<64>(St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
         case 128: return launch_search128(St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
         case 96: return search_n<96>(St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
-        case 160: return search_n<160>(St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
-        case 200: return launch_search_n200(St, T, Sp, degen, P, keys, peaks_all, num_sms, st, nullptr, 0);
+        case 160:
+        case 200: return launch_search_lines(N, St, T, Sp, degen, P, keys, peaks_all, num_sms, st, nullptr, 0);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -724,8 +724,8 @@ cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc,
         case 64: return search_n<64>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         case 128: return search_n<128>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         case 96: return search_n<96>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
-        case 160: return search_n<160>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
-        case 200: return launch_search_n200(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
+        case 160:
+        case 200: return launch_search_lines(N, St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         default: return cudaErrorInvalidValue;
     }
 }

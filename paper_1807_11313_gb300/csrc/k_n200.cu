@@ -1,29 +1,29 @@
-// The native 200 x 200 detector side: pre-processing, the all-pairs search
-// and the single-surface peak.
+// The native 200 x 200 detector side: pre-processing and the single-surface
+// peak (the all-pairs search is in k_lines.cu).
 //
 // Paper: FFT section (Eq. 4 transform, window, band-pass, normalisation by the
 // autocorrelations; footnote 1: the crop to 2^n only makes the transform and
 // the filters easier, so a 200 px detector can be used whole), Eqs. 3 and 6
 // (the correlation surface), the peak fit of Fig. 1 C.
 //
-// The complex 200 x 200 array of two packed surfaces (320 KB) fits no SM, so
-// one template is correlated at a time through the real-output inverse
-// transform, whose working array is the 200 x 101 half spectrum (162 KB, in
-// shared memory): X = conj(S_t) S_p over the stored half (u < 200, v <= 100);
-// the 101 columns are inverse-transformed over u (200 points); each row y
-// then goes back to 200 real values through one 100-point complex transform,
-// z[k] = E[k] + i O[k] with E[k] = C[k] + conj C[100 - k] and O[k] =
-// (C[k] - conj C[100 - k]) e^{+2 pi i k / 200}, whose real and imaginary
-// parts are the even and odd columns of the surface.  The pre-processing runs
-// the same steps forwards (rows as 100-point transforms of (x[2n], x[2n+1])
-// split into the 101-point half row, then the columns) and, for the filtered
-// image, backwards.
+// The complex 200 x 200 array (320 KB) fits no SM, so both go through the
+// real-input / real-output transform, whose working array is the 200 x 101 half
+// spectrum (162 KB, in shared memory).  The peak: X = conj(S_t) S_p over the
+// stored half (u < 200, v <= 100); the 101 columns are inverse-transformed over
+// u (200 points); each row y then goes back to 200 real values through one
+// 100-point complex transform, z[k] = E[k] + i O[k] with E[k] = C[k] + conj
+// C[100 - k] and O[k] = (C[k] - conj C[100 - k]) e^{+2 pi i k / 200}, whose real
+// and imaginary parts are the even and odd columns of the surface.  The
+// pre-processing runs the same steps forwards (rows as 100-point transforms of
+// (x[2n], x[2n+1]) split into the 101-point half row, then the columns) and, for
+// the filtered image, backwards.
 //
 // Line transforms: one warp per line, Stockham autosort passes in shared
 // memory between two per-warp line buffers, radices 8, 5, 5 (200 points) and
 // 4, 5, 5 (100 points), the small DFTs in registers, the twiddles from one
 // table of e^{+2 pi i e / 200}.
 #include "common.cuh"
+#include "dft_small.cuh"
 #include "generic.cuh"
 #include "kernels.cuh"
 
@@ -55,28 +55,6 @@ __device__ __forceinline__ void dft4(float2 (&v)[4]) {
     v[1] = c_add(d02, d13);
     v[3] = c_sub(d02, d13);
 }
-// radix 5 from the sums and differences of the conjugate-symmetric pairs
-// (v1, v4) and (v2, v3): V_1,4 = v0 + c1 t1 + c2 t2 +- i SIGN (s1 t3 + s2 t4),
-// V_2,3 = v0 + c2 t1 + c1 t2 +- i SIGN (s2 t3 - s1 t4)
-template <int SIGN>
-__device__ __forceinline__ void dft5(float2 (&v)[5]) {
-    constexpr float c1 = Tw<1, 5, +1>::re, s1 = Tw<1, 5, +1>::im;
-    constexpr float c2 = Tw<2, 5, +1>::re, s2 = Tw<2, 5, +1>::im;
-    const float2 t1 = c_add(v[1], v[4]), t2 = c_add(v[2], v[3]);
-    const float2 t3 = c_sub(v[1], v[4]), t4 = c_sub(v[2], v[3]);
-    const float2 a1 = make_float2(fmaf(c1, t1.x, fmaf(c2, t2.x, v[0].x)), fmaf(c1, t1.y, fmaf(c2, t2.y, v[0].y)));
-    const float2 a2 = make_float2(fmaf(c2, t1.x, fmaf(c1, t2.x, v[0].x)), fmaf(c2, t1.y, fmaf(c1, t2.y, v[0].y)));
-    float2 b1 = make_float2(fmaf(s1, t3.x, s2 * t4.x), fmaf(s1, t3.y, s2 * t4.y));
-    float2 b2 = make_float2(fmaf(s2, t3.x, -s1 * t4.x), fmaf(s2, t3.y, -s1 * t4.y));
-    // i SIGN b
-    b1 = SIGN > 0 ? c_mul_pi(b1) : c_mul_mi(b1);
-    b2 = SIGN > 0 ? c_mul_pi(b2) : c_mul_mi(b2);
-    v[0] = c_add(v[0], c_add(t1, t2));
-    v[1] = c_add(a1, b1);
-    v[4] = c_sub(a1, b1);
-    v[2] = c_add(a2, b2);
-    v[3] = c_sub(a2, b2);
-}
 template <int SIGN>
 __device__ __forceinline__ void dft8(float2 (&v)[8]) {
     fft_reg_dif<8, SIGN>(v);   // v[p] = V[bitrev3(p)]
@@ -89,7 +67,7 @@ __device__ __forceinline__ void dft8(float2 (&v)[8]) {
 template <int R, int SIGN>
 __device__ __forceinline__ void dft(float2 (&v)[R]) {
     if constexpr (R == 4) dft4<SIGN>(v);
-    else if constexpr (R == 5) dft5<SIGN>(v);
+    else if constexpr (R == 5) ::dft::dft5<SIGN>(v[0], v[1], v[2], v[3], v[4]);
     else dft8<SIGN>(v);
 }
 
@@ -259,64 +237,6 @@ __global__ void __launch_bounds__(NT, 1) k_prep_n200(const float *__restrict__ i
     }
 }
 
-// ------------------------------------------------------------------- search
-// pattern p (blockIdx.y) against the slots [jb, je) (every template, or the
-// pattern's candidate list); one template per pass; the best into keys[p]
-__global__ void __launch_bounds__(NT, 1) k_search_n200(const float2 *__restrict__ St, int T,
-                                                       const float2 *__restrict__ Sp, const int *__restrict__ degen,
-                                                       int per_cta, unsigned long long *__restrict__ keys,
-                                                       float *__restrict__ peaks_all, const int *__restrict__ cand,
-                                                       int kc) {
-    const int p = blockIdx.y;
-    if (degen[p]) return;
-    const int n = cand ? kc : T;
-    const int jb = blockIdx.x * per_cta, je = min(n, jb + per_cta);
-    if (jb >= je) return;
-    extern __shared__ float4 smem_raw[];
-    float2 *buf = reinterpret_cast<float2 *>(smem_raw);
-    float2 *tw = buf + OFF_TW;
-    __shared__ float rmax[NWARP];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float2 *sa = buf + OFF_SCR + warp * 2 * N, *sb = sa + N;
-    make_tw200(tw);
-    const float2 *sp = Sp + (size_t)p * N * HW;
-    float best_v = -INFINITY;
-    int best_t = -1;
-    for (int j = jb; j < je; ++j) {
-        const int t = cand ? cand[(size_t)p * kc + j] : j;
-        if (t < 0) {   // an empty candidate slot (uniform over the CTA)
-            if (peaks_all && tid == 0) peaks_all[(size_t)p * n + j] = -INFINITY;
-            continue;
-        }
-        const float2 *st = St + (size_t)t * N * HW;
-        __syncthreads();   // the previous template's rows are read; the twiddles are in place
-        for (int it = tid; it < N * HW; it += NT) buf[it] = c_mulcj(__ldg(st + it), __ldg(sp + it));
-        __syncthreads();
-        columns<+1>(buf, sa, sb, tw, warp, lane);
-        __syncthreads();
-        float m = -INFINITY;
-        for (int y = warp; y < N; y += NWARP) {
-            row_c2r(buf, y, sa, sb, tw, lane);
-            for (int k = lane; k < M; k += 32) m = fmaxf(m, fmaxf(sb[k].x, sb[k].y));
-            __syncwarp();
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) rmax[warp] = m;
-        __syncthreads();
-        if (tid == 0) {
-            float v = rmax[0];
-            for (int w = 1; w < NWARP; ++w) v = fmaxf(v, rmax[w]);
-            if (peaks_all) peaks_all[(size_t)p * n + j] = v;
-            if (v > best_v || (v == best_v && t < best_t)) {
-                best_v = v;
-                best_t = t;
-            }
-        }
-    }
-    if (tid == 0 && best_t >= 0) atomicMax(keys + p, pack_key(best_v, best_t));
-}
-
 __device__ __forceinline__ float parabola200(float cm, float c0, float cp) {
     const float den = cm - 2.f * c0 + cp;
     if (!(den < 0.f)) return 0.f;
@@ -426,24 +346,6 @@ cudaError_t launch_prep_n200(const float *img, int P, const PrepArgs &a, float2 
     cudaError_t e = smem_attr(k_prep_n200);
     if (e != cudaSuccess) return e;
     k_prep_n200<<<P, NT, SMEM_BYTES, st>>>(img, a, spec, spatial, degen, active);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_search_n200(const float2 *St, int T, const float2 *Sp, const int *degen, int P,
-                               unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st,
-                               const int *cand, int kc) {
-    const int n = cand ? kc : T;
-    if (P <= 0 || n <= 0) return cudaSuccess;
-    cudaError_t e = smem_attr(k_search_n200);
-    if (e != cudaSuccess) return e;
-    // enough CTAs to fill the GPU twice over, at least 4 templates each
-    const long want = (long)num_sms * 2;
-    int chunks = (int)((want + P - 1) / P);
-    chunks = max(1, min(chunks, (n + 3) / 4));
-    int per = (n + chunks - 1) / chunks;
-    chunks = (n + per - 1) / per;
-    dim3 grid(chunks, P);
-    k_search_n200<<<grid, NT, SMEM_BYTES, st>>>(St, T, Sp, degen, per, keys, peaks_all, cand, kc);
     return cudaGetLastError();
 }
 

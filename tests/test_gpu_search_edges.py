@@ -99,9 +99,9 @@ def test_search_64_and_96(px, n, T, P):
     check_search(px, n, T, P, native=1)
 
 
-@pytest.mark.parametrize("n", [64, 96])
+@pytest.mark.parametrize("n", [64, 96, 160, 200])
 @pytest.mark.parametrize("k", [1, 2, 5, 8])
-def test_candidate_lists_64_and_96(px, n, k):
+def test_candidate_lists(px, n, k):
     """Lists with empty entries, repeated templates (ties to the lowest index)
     and descending order against float64."""
     T, P = 20, 5
@@ -129,3 +129,10 @@ def test_candidate_lists_64_and_96(px, n, k):
         torch.testing.assert_close(peak[p].double(), ref[p, top], rtol=1e-4, atol=1e-6)
     lib.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 7, 8, 9, 17])
+@pytest.mark.parametrize("P", [1, 3])
+@pytest.mark.parametrize("n", [160, 200])
+def test_search_160_and_200(px, n, T, P):
+    check_search(px, n, T, P, native=1)
