@@ -672,7 +672,7 @@ int build_from_master(xcf_ctx *ctx, const float *master, int32_t M, const double
         ctx->launches[XCF_STAGE_PREP] += 1;
     }
     if (spectra && e == cudaSuccess && has_search_layout(c.n)) {
-        e = cudaMalloc(&lib->spectra_pk, sizeof(float2) * search_layout_f2(c.n) * T);
+        e = cudaMalloc(&lib->spectra_pk, sizeof(float2) * H * T);
         if (e == cudaSuccess) e = launch_pack_search_layout(lib->spectra, T, c.n, lib->spectra_pk, st);
         ctx->launches[XCF_STAGE_OTHER] += 1;
     }
@@ -727,7 +727,7 @@ int build_from_images(xcf_ctx *ctx, const float *images, const double *quats, in
         ctx->launches[XCF_STAGE_PREP] += 1;
     }
     if (spectra && e == cudaSuccess && has_search_layout(c.n)) {
-        e = cudaMalloc(&lib->spectra_pk, sizeof(float2) * search_layout_f2(c.n) * T);
+        e = cudaMalloc(&lib->spectra_pk, sizeof(float2) * H * T);
         if (e == cudaSuccess) e = launch_pack_search_layout(lib->spectra, T, c.n, lib->spectra_pk, st);
         ctx->launches[XCF_STAGE_OTHER] += 1;
     }

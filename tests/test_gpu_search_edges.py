@@ -99,7 +99,7 @@ def test_search_64_and_96(px, n, T, P):
     check_search(px, n, T, P, native=1)
 
 
-@pytest.mark.parametrize("n", [64, 96, 160, 200])
+@pytest.mark.parametrize("n", [64, 96, 160, 200, 256])
 @pytest.mark.parametrize("k", [1, 2, 5, 8])
 def test_candidate_lists(px, n, k):
     """Lists with empty entries, repeated templates (ties to the lowest index)
@@ -136,3 +136,9 @@ def test_candidate_lists(px, n, k):
 @pytest.mark.parametrize("n", [160, 200])
 def test_search_160_and_200(px, n, T, P):
     check_search(px, n, T, P, native=1)
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 17, 65])
+@pytest.mark.parametrize("P", [1, 3, 80])
+def test_search_256(px, T, P):
+    check_search(px, 256, T, P)
