@@ -405,8 +405,8 @@ int refine_chunk(xcf_ctx *ctx, const xcf_library *lib, const float *patterns, in
                    launch_logpolar(yt, active, P, n, r.nr, r.neta, (float)r.rmin, (float)r.rmax, lpt, st),
                    "logpolar templates");
         XCF_LAUNCH(XCF_STAGE_UPDATE, st,
-                   launch_eta_update(lpt, lpp, r.nr, r.neta, r.windows, quats, q1, alpha, tol_deg, active, iters,
-                                     quats, P, st),
+                   launch_eta_update(lpt, lpp, r.nr, r.neta, r.windows, quats, q1, alpha, tol_deg,
+                                     reinterpret_cast<double *>(shift), active, iters, quats, P, st),   // shift is spent
                    "z update");
     }
     return XCF_OK;

@@ -92,17 +92,22 @@ struct LpPos {
     int o;
     float tx, ty;
 };
-__device__ __forceinline__ LpPos lp_pos(int idx, int N, int nr, int neta, float rmin, float lr) {
+__device__ __forceinline__ float lp_radius(int m, int nr, float rmin, float lr) {
+    return rmin * expf(lr * (nr > 1 ? (float)m / (nr - 1) : 0.f));
+}
+__device__ __forceinline__ LpPos lp_at(float r, float sn, float cs, int N) {
     const float c = 0.5f * N - 0.5f;
-    const int m = idx / neta, l = idx % neta;
-    const float r = rmin * expf(lr * (nr > 1 ? (float)m / (nr - 1) : 0.f));
-    float sn, cs;
-    sincospif(2.f * l / neta, &sn, &cs);
     const float fx = c + r * cs, fy = c - r * sn;
     int x0 = (int)floorf(fx), y0 = (int)floorf(fy);
     x0 = min(max(x0, 0), N - 2);
     y0 = min(max(y0, 0), N - 2);
     return LpPos{y0 * N + x0, fx - x0, fy - y0};
+}
+__device__ __forceinline__ LpPos lp_pos(int idx, int N, int nr, int neta, float rmin, float lr) {
+    const int m = idx / neta, l = idx % neta;
+    float sn, cs;
+    sincospif(2.f * l / neta, &sn, &cs);
+    return lp_at(lp_radius(m, nr, rmin, lr), sn, cs, N);
 }
 __device__ __forceinline__ float lp_bilinear(const float *g, int N, const LpPos &q) {
     return (1.f - q.ty) * ((1.f - q.tx) * g[0] + q.tx * g[1]) + q.ty * ((1.f - q.tx) * g[N] + q.tx * g[N + 1]);
@@ -127,8 +132,11 @@ __global__ void __launch_bounds__(256) k_logpolar(const float *__restrict__ spat
 
 // sides up to kLpSmemSide: one image per CTA, read from HBM once with
 // coalesced 16-byte loads into shared memory and sampled there (the samples'
-// scattered bilinear reads then cost shared-memory wavefronts, not sectors)
-constexpr int kLpSmemSide = 160;
+// scattered bilinear reads then cost shared-memory wavefronts, not sectors).
+// A thread keeps its angles, so that sine and cosine are evaluated once per
+// angle and the radius's exponential once per CTA instead of per sample:
+// 107 -> 62 us per 2,000 images at 128 (32 radii, 256 angles).
+constexpr int kLpSmemSide = 160, kLpMaxRadii = 128;
 __global__ void __launch_bounds__(256) k_logpolar_img(const float *__restrict__ spatial,
                                                       const int *__restrict__ active, int N, int nr, int neta,
                                                       float rmin, float rmax, float *__restrict__ out) {
@@ -136,39 +144,30 @@ __global__ void __launch_bounds__(256) k_logpolar_img(const float *__restrict__ 
     const int p = blockIdx.x;
     if (active && !active[p]) return;
     const float4 *src = reinterpret_cast<const float4 *>(spatial + (size_t)p * N * N);
+    __shared__ float radius[kLpMaxRadii];
+    const float lr = logf(rmax / rmin);
+    if (nr <= kLpMaxRadii && threadIdx.x < nr) radius[threadIdx.x] = lp_radius(threadIdx.x, nr, rmin, lr);
+#pragma unroll 4
     for (int i = threadIdx.x; i < N * N / 4; i += blockDim.x) lp_img4[i] = src[i];
     __syncthreads();
     const float *img = reinterpret_cast<const float *>(lp_img4);
-    const float lr = logf(rmax / rmin);
     float *dst = out + (size_t)p * nr * neta;
+    if (nr <= kLpMaxRadii) {
+        for (int l = threadIdx.x; l < neta; l += blockDim.x) {
+            float sn, cs;
+            sincospif(2.f * l / neta, &sn, &cs);
+#pragma unroll 4
+            for (int m = 0; m < nr; ++m) {
+                const LpPos q = lp_at(radius[m], sn, cs, N);
+                dst[(size_t)m * neta + l] = lp_bilinear(img + q.o, N, q);
+            }
+        }
+        return;
+    }
     for (int idx = threadIdx.x; idx < nr * neta; idx += blockDim.x) {
         const LpPos q = lp_pos(idx, N, nr, neta, rmin, lr);
         dst[idx] = lp_bilinear(img + q.o, N, q);
     }
-}
-
-// means of two FP32 partials per thread over n values: warp sums in FP32, the
-// warps' sums and the division in FP64 by thread 0 alone (GB300's FP64 pipe is
-// narrow); sh: one entry per warp, and one for the result
-__device__ float2 block_means(float a, float b, int n, float2 *sh) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if (lane == 0) sh[w] = make_float2(a, b);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0, t = 0.0;
-        for (int k = 0; k < nw; ++k) {
-            s += (double)sh[k].x;
-            t += (double)sh[k].y;
-        }
-        sh[nw] = make_float2((float)(s / n), (float)(t / n));
-    }
-    __syncthreads();
-    return sh[nw];
 }
 
 __device__ __forceinline__ float parabola(float cm, float c0, float cp) {
@@ -181,30 +180,70 @@ __device__ __forceinline__ float parabola(float cm, float c0, float cp) {
 // ------------------------------------------------ angular correlation + Z
 // c(D) = sum_m sum_l a[m][l] b[m][(l + D) mod neta] / (|a| |b|) on mean-free
 // log-polar images (a = template, b = pattern), by the correlation theorem:
-// each warp transforms radii m = warp, warp + 8, ... as one complex line
-// z = a_m + i b_m, splits A_m and B_m by Hermitian symmetry and accumulates
-// C[k] = sum_m conj(A_m[k]) B_m[k] (k <= neta/2) in registers; the warps'
-// eight sums are added and one inverse transform of the Hermitian C
+// each warp transforms radii m = m0 + warp, m0 + warp + 8, ... of a window as one
+// complex line z = a_m + i b_m, splits A_m and B_m by Hermitian symmetry and
+// accumulates C[k] = sum_m conj(A_m[k]) B_m[k] (k <= neta/2) in registers; the
+// warps' eight sums are added and one inverse transform of the Hermitian C
 // gives c(D) for every shift.  neta log neta work per radius instead of neta^2.
+//
+// Bound by the latency of its chain, so windows go G at a time: their means in
+// one reduction, their lines without a barrier between them, and their inverse
+// transforms side by side on G warps (one window after another, with seven
+// warps waiting for the inverse, and the float64 update at the CTA's end: 280 us
+// per 2,000 patterns at 256 angles; now 150 and 20 for the update kernels).
 constexpr int kEtaThreads = 256, kEtaWarps = kEtaThreads / 32, kMaxLpWindows = 16;
+// windows side by side, by what the warps' sums take in shared memory (48 KB)
+template <int NETA>
+__host__ __device__ constexpr int eta_group() { return NETA >= 512 ? 2 : 4; }
+
+// means of NW pairs of FP32 partials per thread over n[i] values: warp sums in
+// FP32, the warps' sums and the division in FP64 by one thread per pair (GB300's
+// FP64 pipe is narrow); sh: [NW][kEtaWarps + 1]
+template <int NW>
+__device__ __forceinline__ void eta_means(float (&a)[NW], float (&b)[NW], const int (&n)[NW],
+                                          float2 (&sh)[NW][kEtaWarps + 1]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
+            b[i] += __shfl_xor_sync(0xffffffffu, b[i], o);
+        }
+        if (lane == 0) sh[i][w] = make_float2(a[i], b[i]);
+    }
+    __syncthreads();
+    if (lane == 0 && w < NW) {
+        int nw = 0;   // n[w], by constant indexes
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            if (i == w) nw = n[i];
+        double s = 0.0, t = 0.0;
+        for (int k = 0; k < kEtaWarps; ++k) {
+            s += (double)sh[w][k].x;
+            t += (double)sh[w][k].y;
+        }
+        sh[w][kEtaWarps] = nw > 0 ? make_float2((float)(s / nw), (float)(t / nw)) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NW; ++i) a[i] = sh[i][kEtaWarps].x, b[i] = sh[i][kEtaWarps].y;
+}
 
 template <int NETA>
 __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update(const float *__restrict__ lpT,
                                                             const float *__restrict__ lpP, int nr, int windows,
-                                                            const double *__restrict__ q0s,
-                                                            const double *__restrict__ q1s,
-                                                            double alpha, double tol_deg,
-                                                            int *__restrict__ active,
-                                                            int *__restrict__ iters,
-                                                            double *__restrict__ q_out) {
-    constexpr int H = NETA / 2 + 1, KPL = (H + 31) / 32;   // spectrum bins, bins per lane
+                                                            const int *__restrict__ active,
+                                                            double *__restrict__ deta_out) {
+    constexpr int H = NETA / 2 + 1, KPL = (H + 31) / 32, G = eta_group<NETA>();   // spectrum bins, bins per lane
     const int p = blockIdx.x;
     if (!active[p]) return;
-    __shared__ float2 line[kEtaWarps][NETA];   // per-warp lines, then per-warp sums C (k < H)
+    extern __shared__ float4 eta_smem[];
+    // per-warp lines [8][NETA], then the warps' sums [G][8][H] beside them, the G windows' lines [G][NETA]
+    float2 *lines = reinterpret_cast<float2 *>(eta_smem);
+    float2 *sums = lines + kEtaWarps * NETA;
     __shared__ float2 tw[NETA / 2], twi[NETA / 2];
-    __shared__ float2 zc[NETA];
-    __shared__ float cfin[NETA];
-    __shared__ float2 red[kEtaWarps + 1];
+    __shared__ float2 red[G][kEtaWarps + 1];
     __shared__ double wshift[kMaxLpWindows];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const float *ga = lpT + (size_t)p * nr * NETA, *gb = lpP + (size_t)p * nr * NETA;
@@ -214,63 +253,79 @@ __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update
     constexpr bool kRegLine = NETA >= 64;   // register warp transforms (NETA = R x 32)
     WarpFftTw<kRegLine ? NETA : 64> wf;
     if constexpr (kRegLine) wf.load(tw, lane);
-    float2 *z = line[w];
+    float2 *z = lines + w * NETA;
     // radial window b holds radii [b nr / W, (b + 1) nr / W); each is correlated along eta on its own
-    for (int b = 0; b < windows; ++b) {
-        const int m0 = b * nr / windows, m1 = (b + 1) * nr / windows;
-        const int i0 = m0 * NETA, i1 = m1 * NETA;
-        float s1 = 0.f, s2 = 0.f;
-        for (int i = i0 + tid; i < i1; i += kEtaThreads) { s1 += ga[i]; s2 += gb[i]; }
-        const float2 mean = block_means(s1, s2, i1 - i0, red);
-        const float ma = mean.x, mb = mean.y;
-        float2 acc[KPL];
+    for (int b0 = 0; b0 < windows; b0 += G) {
+        float ma[G], mb[G];
+        int n[G];
 #pragma unroll
-        for (int j = 0; j < KPL; ++j) acc[j] = make_float2(0.f, 0.f);
-        for (int m = m0 + w; m < m1; m += kEtaWarps) {
-            // forward: Z[k] = sum_l z[l] e^{-2 pi i k l / NETA}
-            if constexpr (kRegLine) {   // in registers (NETA / 32 points per lane), spectrum to z
-                float2 v[NETA / 32];
+        for (int i = 0; i < G; ++i) {
+            const int b = b0 + i, i0 = b < windows ? b * nr / windows * NETA : 0, i1 = b < windows ? (b + 1) * nr / windows * NETA : 0;
+            ma[i] = mb[i] = 0.f;
+            n[i] = i1 - i0;
+            for (int k = i0 + tid; k < i1; k += kEtaThreads) {
+                ma[i] += ga[k];
+                mb[i] += gb[k];
+            }
+        }
+        eta_means<G>(ma, mb, n, red);
 #pragma unroll
-                for (int j = 0; j < NETA / 32; ++j) {
-                    const size_t i = (size_t)m * NETA + lane + 32 * j;
-                    v[j] = make_float2(ga[i] - ma, gb[i] - mb);
+        for (int i = 0; i < G; ++i) {
+            const int b = b0 + i;
+            if (b >= windows) break;   // uniform
+            const int m0 = b * nr / windows, m1 = (b + 1) * nr / windows;
+            float2 acc[KPL];
+#pragma unroll
+            for (int j = 0; j < KPL; ++j) acc[j] = make_float2(0.f, 0.f);
+            for (int m = m0 + w; m < m1; m += kEtaWarps) {
+                // forward: Z[k] = sum_l z[l] e^{-2 pi i k l / NETA}
+                if constexpr (kRegLine) {   // in registers (NETA / 32 points per lane), spectrum to z
+                    float2 v[NETA / 32];
+#pragma unroll
+                    for (int j = 0; j < NETA / 32; ++j) {
+                        const size_t k = (size_t)m * NETA + lane + 32 * j;
+                        v[j] = make_float2(ga[k] - ma[i], gb[k] - mb[i]);
+                    }
+                    warp_fft_core<NETA>(v, wf, lane);
+#pragma unroll
+                    for (int j = 0; j < NETA / 32; ++j) z[warp_fft_out<NETA>(lane, j)] = v[j];
+                    __syncwarp();
+                } else {
+                    for (int l = lane; l < NETA; l += 32)
+                        z[l] = make_float2(ga[(size_t)m * NETA + l] - ma[i], gb[(size_t)m * NETA + l] - mb[i]);
+                    __syncwarp();
+                    linefft::warp_fft_line<NETA>(z, 1, tw);
                 }
-                warp_fft_core<NETA>(v, wf, lane);
 #pragma unroll
-                for (int j = 0; j < NETA / 32; ++j) z[warp_fft_out<NETA>(lane, j)] = v[j];
+                for (int j = 0; j < KPL; ++j) {
+                    const int k = lane + 32 * j;
+                    if (k < H) {
+                        const float2 zk = z[k], zn = z[(NETA - k) & (NETA - 1)];
+                        // A = (Z[k] + conj Z[-k]) / 2, B = (Z[k] - conj Z[-k]) / (2i); acc += conj(A) B
+                        const float2 A = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
+                        const float2 B = make_float2(0.5f * (zk.y + zn.y), 0.5f * (zn.x - zk.x));
+                        acc[j].x += A.x * B.x + A.y * B.y;
+                        acc[j].y += A.x * B.y - A.y * B.x;
+                    }
+                }
                 __syncwarp();
-            } else {
-                for (int l = lane; l < NETA; l += 32)
-                    z[l] = make_float2(ga[(size_t)m * NETA + l] - ma, gb[(size_t)m * NETA + l] - mb);
-                __syncwarp();
-                linefft::warp_fft_line<NETA>(z, 1, tw);
             }
 #pragma unroll
             for (int j = 0; j < KPL; ++j) {
                 const int k = lane + 32 * j;
-                if (k < H) {
-                    const float2 zk = z[k], zn = z[(NETA - k) & (NETA - 1)];
-                    // A = (Z[k] + conj Z[-k]) / 2, B = (Z[k] - conj Z[-k]) / (2i); acc += conj(A) B
-                    const float2 A = make_float2(0.5f * (zk.x + zn.x), 0.5f * (zk.y - zn.y));
-                    const float2 B = make_float2(0.5f * (zk.y + zn.y), 0.5f * (zn.x - zk.x));
-                    acc[j].x += A.x * B.x + A.y * B.y;
-                    acc[j].y += A.x * B.y - A.y * B.x;
-                }
+                if (k < H) sums[(i * kEtaWarps + w) * H + k] = acc[j];
             }
-            __syncwarp();
-        }
-#pragma unroll
-        for (int j = 0; j < KPL; ++j) {
-            const int k = lane + 32 * j;
-            if (k < H) z[k] = acc[j];
         }
         __syncthreads();
-        // C[k] over the warps in float64, extended by C[NETA - k] = conj C[k]; inverse transform by warp 0.
-        // The correlation's scale does not move its argmax or parabolic offset, so it is not normalised.
-        if (w == 0) {
+        // window b0 + w on warp w < G: C[k] over the warps, extended by C[NETA - k] = conj C[k], and its
+        // inverse transform.  The correlation's scale does not move its argmax or parabolic offset, so it
+        // is not normalised.
+        if (w < G && b0 + w < windows) {
+            const float2 *cw = sums + w * kEtaWarps * H;
+            float2 *zc = z;
             for (int k = lane; k < H; k += 32) {
                 float cr = 0.f, ci = 0.f;   // eight FP32 partials (FP64 here kept GB300's narrow FP64 pipe busy)
-                for (int v = 0; v < kEtaWarps; ++v) { cr += line[v][k].x; ci += line[v][k].y; }
+                for (int v = 0; v < kEtaWarps; ++v) { cr += cw[v * H + k].x; ci += cw[v * H + k].y; }
                 zc[k] = make_float2(cr, ci);
                 if (k > 0 && k < NETA / 2) zc[NETA - k] = make_float2(cr, -ci);
             }
@@ -283,27 +338,26 @@ __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update
                 for (int j = 0; j < NETA / 32; ++j) v[j] = zc[lane + 32 * j];
                 warp_fft_core<NETA>(v, wi, lane);
 #pragma unroll
-                for (int j = 0; j < NETA / 32; ++j) cfin[warp_fft_out<NETA>(lane, j)] = v[j].x;
+                for (int j = 0; j < NETA / 32; ++j) zc[warp_fft_out<NETA>(lane, j)].x = v[j].x;
             } else {
                 linefft::warp_fft_line<NETA>(zc, 1, twi);
-                for (int d = lane; d < NETA; d += 32) cfin[d] = zc[d].x;
             }
             __syncwarp();
             // argmax over the shifts (the lowest shift among equal maxima), then the parabola
             int best = lane;
             for (int D = lane + 32; D < NETA; D += 32)
-                if (cfin[D] > cfin[best]) best = D;
+                if (zc[D].x > zc[best].x) best = D;
 #pragma unroll
             for (int o = 16; o; o >>= 1) {
                 const int ob = __shfl_xor_sync(0xffffffffu, best, o);
-                if (cfin[ob] > cfin[best] || (cfin[ob] == cfin[best] && ob < best)) best = ob;
+                if (zc[ob].x > zc[best].x || (zc[ob].x == zc[best].x && ob < best)) best = ob;
             }
             if (lane == 0) {
-                const float off = parabola(cfin[(best + NETA - 1) % NETA], cfin[best], cfin[(best + 1) % NETA]);
-                wshift[b] = (double)(best < NETA / 2 ? best : best - NETA) + off;
+                const float off = parabola(zc[(best + NETA - 1) % NETA].x, zc[best].x, zc[(best + 1) % NETA].x);
+                wshift[b0 + w] = (double)(best < NETA / 2 ? best : best - NETA) + off;
             }
         }
-        __syncthreads();   // line, zc and cfin are reused by the next window
+        __syncthreads();   // lines and sums are reused by the next windows
     }
     if (tid == 0) {
         // median of the window shifts (mean of the middle two for an even count)
@@ -313,20 +367,35 @@ __global__ void __launch_bounds__(kEtaThreads, NETA >= 512 ? 2 : 3) k_eta_update
                 wshift[j] = wshift[j - 1];
                 wshift[j - 1] = t;
             }
-        const double deta = windows % 2 ? wshift[windows / 2] : 0.5 * (wshift[windows / 2 - 1] + wshift[windows / 2]);
-        const double tz = 2.0 * XCF_PI * deta / NETA;
-        double s, c;
-        sincos(0.5 * tz, &s, &c);
-        const Q Rz = {c, 0.0, 0.0, s};
-        const Q q0 = qload(q0s + 4 * (size_t)p);
-        const Q q2 = rotate_in_detector(qload(q1s + 4 * (size_t)p), Rz, alpha);
-        double dot = fabs(q2.w * q0.w + q2.x * q0.x + q2.y * q0.y + q2.z * q0.z);
-        dot = fmin(dot, 1.0);
-        const double upd = 2.0 * acos(dot) * 180.0 / XCF_PI;
-        qstore(q_out + 4 * (size_t)p, q2);
-        iters[p] += 1;
-        if (upd < tol_deg) active[p] = 0;
+        deta_out[p] = windows % 2 ? wshift[windows / 2] : 0.5 * (wshift[windows / 2 - 1] + wshift[windows / 2]);
     }
+}
+
+// the float64 updates, one thread per pattern on one-warp CTAs: a few hundred
+// dependent FP64 operations each, so they are spread over the SMs' narrow FP64
+// pipes, and are not the tail of a correlation CTA (40 us of it)
+constexpr int kUpdateThreads = 32;
+
+// the angular shift as a rotation about the detector z axis; convergence
+__global__ void __launch_bounds__(kUpdateThreads) k_update_z(const double *__restrict__ deta, int neta,
+                                                             const double *__restrict__ q0s,
+                                                             const double *__restrict__ q1s, double alpha,
+                                                             double tol_deg, int P, int *__restrict__ active,
+                                                             int *__restrict__ iters, double *__restrict__ q_out) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= P || !active[p]) return;
+    const double tz = 2.0 * XCF_PI * deta[p] / neta;
+    double s, c;
+    sincos(0.5 * tz, &s, &c);
+    const Q Rz = {c, 0.0, 0.0, s};
+    const Q q0 = qload(q0s + 4 * (size_t)p);
+    const Q q2 = rotate_in_detector(qload(q1s + 4 * (size_t)p), Rz, alpha);
+    double dot = fabs(q2.w * q0.w + q2.x * q0.x + q2.y * q0.y + q2.z * q0.z);
+    dot = fmin(dot, 1.0);
+    const double upd = 2.0 * acos(dot) * 180.0 / XCF_PI;
+    qstore(q_out + 4 * (size_t)p, q2);
+    iters[p] += 1;
+    if (upd < tol_deg) active[p] = 0;
 }
 
 __global__ void k_update_xy(const double *__restrict__ qs, const float *__restrict__ shift,
@@ -484,20 +553,23 @@ cudaError_t launch_update_xy(const double *q, const float *shift, const double *
                              int W, double alpha, const int *active, int P, double *q1,
                              cudaStream_t st) {
     if (P <= 0) return cudaSuccess;
-    k_update_xy<<<(P + 127) / 128, 128, 0, st>>>(q, shift, pcs, pcz_def, W, alpha, active, P, q1);
+    k_update_xy<<<(P + kUpdateThreads - 1) / kUpdateThreads, kUpdateThreads, 0, st>>>(q, shift, pcs, pcz_def, W, alpha, active, P, q1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_eta_update(const float *lpT, const float *lpP, int nr, int neta, int windows,
-                              const double *q0, const double *q1, double alpha, double tol_deg, int *active,
-                              int *iters, double *q_out, int P, cudaStream_t st) {
+                              const double *q0, const double *q1, double alpha, double tol_deg, double *deta,
+                              int *active, int *iters, double *q_out, int P, cudaStream_t st) {
     if (P <= 0) return cudaSuccess;
     if (windows < 1 || windows > kMaxLpWindows || windows > nr) return cudaErrorInvalidValue;
-#define XCF_ETA_CASE(NE)                                                                                    \
-    case NE:                                                                                                \
-        k_eta_update<NE><<<P, kEtaThreads, 0, st>>>(lpT, lpP, nr, windows, q0, q1, alpha, tol_deg, active,   \
-                                                    iters, q_out);                                          \
-        break;
+#define XCF_ETA_CASE(NE)                                                                                     \
+    case NE: {                                                                                               \
+        const int sm = (int)sizeof(float2) * (kEtaWarps * NE + eta_group<NE>() * kEtaWarps * (NE / 2 + 1));  \
+        cudaError_t e = cudaFuncSetAttribute(k_eta_update<NE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); \
+        if (e != cudaSuccess) return e;                                                                      \
+        k_eta_update<NE><<<P, kEtaThreads, sm, st>>>(lpT, lpP, nr, windows, active, deta);                   \
+        break;                                                                                               \
+    }
     switch (neta) {
         XCF_ETA_CASE(32)
         XCF_ETA_CASE(64)
@@ -507,6 +579,8 @@ cudaError_t launch_eta_update(const float *lpT, const float *lpP, int nr, int ne
         default: return cudaErrorInvalidValue;   // neta = 2N for N = 16 .. 256
     }
 #undef XCF_ETA_CASE
+    k_update_z<<<(P + kUpdateThreads - 1) / kUpdateThreads, kUpdateThreads, 0, st>>>(deta, neta, q0, q1, alpha, tol_deg,
+                                                                                     P, active, iters, q_out);
     return cudaGetLastError();
 }
 

@@ -157,9 +157,10 @@ cudaError_t launch_update_xy(const double *q, const float *shift, const double *
                              cudaStream_t st);
 // windows: radial bands of the log-polar images (1 .. min(16, nr)), each
 // correlated along eta on its own; the update takes the median band shift
+// (deta [P]: work array)
 cudaError_t launch_eta_update(const float *lpT, const float *lpP, int nr, int neta, int windows,
-                              const double *q0, const double *q1, double alpha, double tol_deg, int *active,
-                              int *iters, double *q_out, int P, cudaStream_t st);
+                              const double *q0, const double *q1, double alpha, double tol_deg, double *deta,
+                              int *active, int *iters, double *q_out, int P, cudaStream_t st);
 
 cudaError_t launch_gather_seeds(const double *lib_quats, const int *best, int P, double *seeds,
                                 cudaStream_t st);
