@@ -358,7 +358,7 @@ int xcf_nearest_disorientation(xcf_ctx *ctx, const double *qa, int32_t na, const
  * native rule).  Patterns are pre-processed per map, then every map up to
  * 160 x 160 is searched in ONE persistent launch (one 512-thread CTA per SM)
  * that takes (map, pattern, template range) work items of all sides from one
- * queue; 256 x 256 maps (four-CTA clusters) and native 200 x 200 maps (one
+ * queue; 256 x 256 maps (thread-block clusters) and native 200 x 200 maps (one
  * template per pass through the real-output transform) run their own search
  * kernels in the same stream.  For each (detector side, library size) the
  * search body and the work granularity are chosen by timing candidates on the

@@ -243,8 +243,8 @@ bool supported_n(int n) {
     return n == 16 || n == 32 || n == 64 || n == 96 || n == 128 || n == 160 || n == 200 || n == 256;
 }
 
-// pre-processing, search and peak: shared-memory kernels up to N = 160, the
-// four-CTA cluster kernels for N = 256
+// pre-processing, search and peak: shared-memory kernels up to N = 200,
+// thread-block clusters (two or four CTAs) for N = 256
 cudaError_t run_prep(xcf_ctx * /*ctx*/, const float *img, int P, const PrepArgs &a, float2 *spec, float *spatial,
                      int *degen, const int *active, cudaStream_t st) {
     if (a.N == 200) return launch_prep_n200(img, P, a, spec, spatial, degen, active, st);
@@ -1901,7 +1901,7 @@ const xcf_ctx::Tuning *tuned(const xcf_ctx *ctx, int N, int T) {
 
 // sides served by the persistent queue: every side up to 160 x 160 (512-thread
 // CTAs, one per SM, with shared memory for the largest body); 256 x 256 needs
-// a four-CTA cluster, so those maps run the cluster kernel in the same stream
+// thread-block clusters, so those maps run the cluster kernel in the same stream
 // (and graph)
 bool queued_side(int N) { return N != 256 && N != 200; }
 

@@ -21,7 +21,7 @@
 // The maps may have different libraries, pattern centres and detectors.  A
 // CTA never waits for another: the queue only hands out indices.  The
 // alternative launch shape (one CTA per item, grid = items) is one of the
-// autotuner's candidates.  (256 x 256 maps need four-CTA clusters and run
+// autotuner's candidates.  (256 x 256 maps need thread-block clusters and run
 // the cluster kernel: see queued_side in api.cu.)
 #include "common.cuh"
 #include "kernels.cuh"

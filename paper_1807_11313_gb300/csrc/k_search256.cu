@@ -23,13 +23,16 @@
 // What bounds it: sixteen warps go through the passes together, and the load
 // queue (64 global and 16 cluster loads per thread and template) fills in the
 // first and third; issue is active 42 %.  300 patterns x 1,018 templates: 53.6 ->
-// 40.8 ms (15.9 -> 21 TFLOP/s, 26 % of the FP32 peak) against template pairs on
-// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.76 ms.
+// 39.7 ms (15.9 -> 22 TFLOP/s, 27 % of the FP32 peak) against template pairs on
+// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.64 ms.  A
+// full release at the barrier between the column and line passes costs 3 % of that
+// (40.8, 4.76).
 // Measured without gain: 16-byte template loads from an aligned copy of the
 // library with half of the pattern in shared memory (41.3), the next template's
 // first values loaded a pass ahead (49.4: spills), 1,024 threads at 64 registers
 // (42.2), all gathers as cluster loads (41.6).  The templates stay in the plain
 // layout: no second copy of the library (5.5 GB at 20,000 templates).
+#include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -44,27 +47,6 @@ struct Smem {
     float red[NT / 32];
     float top[NC];           // CTA 0: the CTAs' maxima of a surface (every-peak mode)
 };
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// without release: orders reads already consumed before it against writes after the wait
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t map_to_rank(const void *p, uint32_t rank) {
-    const uint32_t local = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ float2 ld_cluster(uint32_t addr) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-    return v;
-}
 
 // decimation-in-frequency stages 0 .. 2 of a 16-point inverse transform
 __device__ __forceinline__ void dif16_head(float2 (&x)[16]) {
@@ -223,7 +205,7 @@ k_search256(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp,
                     col[2048 * i + 64] = zm;
                 });
             }
-            cluster_arrive();
+            cluster_arrive_shared();
             cluster_wait();   // both CTAs' columns are complete
             // ---- 3
             float2 z[2][16];
@@ -303,24 +285,10 @@ cudaError_t launch_search_c256(const float2 *St, int T, const float2 *Sp, const 
     const int n = cand ? kc : T;
     if (P <= 0 || n <= 0) return cudaSuccess;
     auto *kern = peaks_all ? k_search256<true> : k_search256<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = sizeof(Smem);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = NC;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(NC * 64);
+    static std::atomic<int> resident[2] = {{0}, {0}};
     int ncl_max = 0;
-    e = cudaOccupancyMaxActiveClusters(&ncl_max, kern, &cfg);
+    const cudaError_t e = resident_clusters(kern, NC, NT, sizeof(Smem), resident[peaks_all ? 1 : 0], &ncl_max);
     if (e != cudaSuccess) return e;
-    if (ncl_max <= 0) return cudaErrorInvalidConfiguration;
     // chunks of templates so that there are at least ~4 items per resident cluster
     const long want = 4L * ncl_max;
     int nchunks = (int)((want + P - 1) / P);
@@ -329,7 +297,6 @@ cudaError_t launch_search_c256(const float2 *St, int T, const float2 *Sp, const 
     nchunks = (n + per - 1) / per;
     const long n_items = (long)P * nchunks;
     if (n_items > (1L << 30)) return cudaErrorInvalidValue;
-    const int ncl = (int)(n_items < ncl_max ? n_items : ncl_max);
-    cfg.gridDim = dim3(NC * ncl);
-    return cudaLaunchKernelEx(&cfg, kern, St, T, Sp, degen, nchunks, per, (int)n_items, keys, peaks_all, cand, kc);
+    return launch_clusters(kern, NC, NT, sizeof(Smem), n_items < ncl_max ? n_items : ncl_max, st, St, T, Sp, degen,
+                           nchunks, per, (int)n_items, keys, peaks_all, cand, kc);
 }

@@ -58,11 +58,11 @@ cudaError_t launch_search(int N, const float2 *St, int T, const float2 *Sp, cons
 cudaError_t launch_search_c256(const float2 *St, int T, const float2 *Sp, const int *degen, int P,
                                unsigned long long *keys, float *peaks_all, const int *cand, int kc,
                                cudaStream_t st);
-// N = 256 single-surface peak on clusters of four CTAs (two patterns per pass)
+// N = 256 single-surface peak on clusters of four CTAs (k_peak256.cu)
 cudaError_t launch_pair_peak_c256(const float2 *St, const int *tidx, const float2 *Sp, const int *degen,
                                   const int *active, int P, float *peak, float *shift, cudaStream_t st,
                                   int *argmax = nullptr);
-// N = 256 pre-processing on clusters of four CTAs (one image per cluster)
+// N = 256 pre-processing on clusters of four CTAs (k_prep256.cu)
 cudaError_t launch_prep_c256(const float *img, int P, const PrepArgs &a, float2 *spec, float *spatial, int *degen,
                              const int *active, cudaStream_t st);
 

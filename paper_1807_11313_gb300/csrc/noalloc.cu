@@ -185,7 +185,7 @@ extern "C" int xcf_index_noalloc(xcf_ctx *ctx, const xcf_library *lib, const flo
     a.inv2shp = (float)(1.0 / (2.0 * shp * shp));
     a.inv2slp = (float)(1.0 / (2.0 * slp * slp));
 
-    // N = 256 runs on four-CTA clusters, which need no scratch beyond the spectra
+    // N = 256 runs on thread-block clusters, which need no scratch beyond the spectra
     const bool c256 = n == 256;
     if ((rc = launch(ctx, XCF_STAGE_PREP, st, [&] {
              return c256 ? launch_prep_c256(patterns, P, a, sp, nullptr, degen, nullptr, st)
