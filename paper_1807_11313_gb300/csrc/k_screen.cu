@@ -8,33 +8,49 @@
 // library cheaply before the FP32 FFT cross-correlation rescores the best k.
 //
 // k_screen_tc: one CTA (128 threads) computes a 128 (patterns) x 256
-// (templates) tile of S.  Warp 0 is the loader: one thread issues TMA
-// (cp.async.bulk.tensor) copies of 64-wide K-slices of both operands into a
-// four-stage ring, 128-byte swizzled, each stage completing an mbarrier by
-// transaction count.  Warp 1 is the tensor-core issuer: one thread waits for
-// a stage, issues four tcgen05.mma (M = 128, N = 256, K = 16, BF16 in, FP32
-// accumulated in 256 TMEM columns) and commits them to the stage's "empty"
-// mbarrier, which hands the stage back to the loader.  After the last commit
-// all four warps read the accumulator with tcgen05.ld (each warp its 32 TMEM
-// lanes = tile rows) and write S.  Tiles are ordered in groups of eight
-// pattern tiles, so that the CTAs resident at one time share the template
-// tiles they stream.  Every wait is bounded: on time-out the kernel records an
-// error flag, waits (bounded) for its copies in flight and frees its tensor
-// memory.
+// (templates) tile of S, or two CTAs a 256 x 256 tile.  Warp 0 is the loader:
+// one thread issues TMA (cp.async.bulk.tensor) copies of 64-wide K-slices of
+// both operands into a ring of stages, 128-byte swizzled, each stage completing
+// an mbarrier by transaction count.  Warp 1 is the tensor-core issuer: one thread
+// waits for a stage, issues four tcgen05.mma (K = 16, BF16 in, FP32 accumulated in
+// 256 TMEM columns) and commits them to the stage's "empty" mbarrier, which hands
+// the stage back to the loader.  After the last commit all four warps read the
+// accumulator with tcgen05.ld (each warp its 32 TMEM lanes = tile rows) and
+// write S.  Tiles are ordered in groups of eight pattern tiles, so that the CTAs
+// resident at one time share the template tiles they stream.  Every wait is
+// bounded: on time-out the kernel records an error flag, waits (bounded) for its
+// copies in flight and frees its tensor memory.
+//
+// What bounds it: shared-memory traffic of the operands with one CTA per tile (per
+// K-slice 48 KB in by TMA and 48 KB out to the tensor core, 768 cycles of the 128
+// bytes a cycle against 512 of MMA).  A pair holds half of the template slice in
+// each CTA (32 KB in and out, 512 cycles): rank 0 issues instructions that read both
+// CTAs' shared memory and write both accumulators; rank 1's second warp passes
+// "stage loaded" on to it, releasing only shared memory (a full release at each
+// stage waits a microsecond: 4.7 ms instead of 1.5).  2,000 patterns x 39,784
+// templates at K = 16,384: 1.88 -> 1.65 ms by storing S through shared memory, a row
+// at a time, -> 1.50 by pairs (1.74 PFLOP/s, 90 % of the measured BF16 burst);
+// 1,000 x 19,944 at K = 65,536: 1.86 -> 1.77 -> 1.65 (5 rounds of tiles for 4.1).
+// Template tiles of 224 there: 1.63, but 1.64 against 1.50 for the former: 256.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4, NT = 128, GROUP_M = 8;
+constexpr int BM = 128, BN = 256, BK = 64, NT = 128, GROUP_M = 8;
 constexpr int A_BYTES = BM * BK * 2;              // 16 KB
-constexpr int B_BYTES = BN * BK * 2;              // 32 KB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;    // 48 KB
-constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 1024 + 128;
 constexpr unsigned kSpinLimit = 1u << 26;         // bounded waits
+
+// CG CTAs work on one tile: 128 CG patterns x 256 templates
+template <int CG>
+struct Ring {
+    static constexpr int STAGE_BYTES = A_BYTES + BN / CG * BK * 2, STAGES = CG == 1 ? 4 : 6;   // 48 or 32 KB
+    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
+};
 
 // shared-memory matrix descriptor of a K-major operand tile written by TMA
 // with 128-byte swizzling: start address, leading byte offset 16 (unused for
@@ -47,15 +63,16 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
 }
 
 // instruction descriptor of kind::f16: D = F32, A = B = BF16, both K-major,
-// N = 256, M = 128
+// N = 256, M = 128 per CTA
+template <int CG>
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                            ((uint32_t)(BM >> 4) << 24);
+                            ((uint32_t)(CG * BM >> 4) << 24);
 
 __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
     for (unsigned spin = 0; spin < kSpinLimit; ++spin) {
         uint32_t done;
         asm volatile(
-            "{\n .reg .pred P;\n mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n selp.b32 %0, 1, 0, P;\n}\n"
+            "{\n .reg .pred P;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n selp.b32 %0, 1, 0, P;\n}\n"
             : "=r"(done)
             : "r"(addr), "r"(parity)
             : "memory");
@@ -75,48 +92,69 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+// arrives on the barrier (of every CTA of the tile) when all MMAs issued so far have completed
+template <int CG>
+__device__ __forceinline__ void commit(uint32_t bar) {
+    if constexpr (CG == 1)
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
+    else
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+            "h"((uint16_t)3));
+}
+
+template <int CG>
 __global__ void __launch_bounds__(NT, 1)
 k_screen_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int P, int T, int K,
             float *__restrict__ S, int *__restrict__ err) {
+    using R = Ring<CG>;
+    constexpr int STAGES = R::STAGES;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t sbase0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const uint32_t sbase = (sbase0 + 1023u) & ~1023u;            // 1024-aligned stages (swizzle atoms)
-    const uint32_t full_bar = sbase + STAGES * STAGE_BYTES;       // STAGES mbarriers: stage loaded
+    const uint32_t full_bar = sbase + STAGES * R::STAGE_BYTES;    // STAGES mbarriers: stage loaded
     const uint32_t empty_bar = full_bar + 8 * STAGES;             // STAGES mbarriers: stage consumed
-    const uint32_t done_bar = empty_bar + 8 * STAGES;             // accumulator complete
+    const uint32_t peer_bar = empty_bar + 8 * STAGES;             // rank 0: STAGES mbarriers: the peer's stage loaded
+    const uint32_t done_bar = peer_bar + 8 * STAGES;              // accumulator complete
     const uint32_t tmem_slot = done_bar + 8;                      // tcgen05.alloc writes here
     unsigned char *gen_base = smem_raw + (sbase - sbase0);
-    volatile uint32_t *tmem_slot_ptr =
-        reinterpret_cast<volatile uint32_t *>(gen_base + STAGES * STAGE_BYTES + 16 * STAGES + 8);
-    volatile int *flag = reinterpret_cast<volatile int *>(gen_base + STAGES * STAGE_BYTES + 16 * STAGES + 16);
+    unsigned char *gen_bars = gen_base + STAGES * R::STAGE_BYTES;
+    volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(gen_bars + 24 * STAGES + 8);
+    volatile int *flag = reinterpret_cast<volatile int *>(gen_bars + 24 * STAGES + 16);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // grouped tile order: GROUP_M pattern tiles per template-tile sweep
-    const int num_m = (P + BM - 1) / BM, num_n = (T + BN - 1) / BN;
-    const int id = blockIdx.x, per_group = GROUP_M * num_n;
-    const int first_m = (id / per_group) * GROUP_M;
-    const int gsize = min(num_m - first_m, GROUP_M);
+    const int rank = CG == 1 ? 0 : (int)cluster_rank();
+    // grouped tile order: GROUP_M / CG pattern tiles per template-tile sweep
+    const int num_m = (P + CG * BM - 1) / (CG * BM), num_n = (T + BN - 1) / BN;
+    const int id = blockIdx.x / CG, per_group = GROUP_M / CG * num_n;
+    const int first_m = (id / per_group) * (GROUP_M / CG);
+    const int gsize = min(num_m - first_m, GROUP_M / CG);
     const int m_tile = first_m + (id % per_group) % gsize, n_tile = (id % per_group) / gsize;
-    const int p0 = m_tile * BM, t0 = n_tile * BN;
+    const int p0 = (m_tile * CG + rank) * BM, t0 = n_tile * BN;   // this CTA's rows of A and of S
     const int nk = K / BK;
 
     if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar + 8 * s));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty_bar + 8 * s));
-        }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(done_bar));
+        for (int s = 0; s < 3 * STAGES + 1; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full_bar + 8 * s));
         asm volatile("fence.mbarrier_init.release.cluster;");
         *flag = 0;
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapA)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapB)) : "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(BN));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        if constexpr (CG == 1) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(BN));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(BN));
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
+    if constexpr (CG == 2) {   // both CTAs' barriers are initialised and their tensor memory allocated
+        cluster_arrive();
+        cluster_wait();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tmem_slot_ptr;
 
@@ -129,36 +167,55 @@ k_screen_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 break;
             }
             if (*flag) break;
-            const uint32_t sa = sbase + s * STAGE_BYTES, sb = sa + A_BYTES;
-            mbar_expect_tx(full_bar + 8 * s, STAGE_BYTES);
+            const uint32_t sa = sbase + s * R::STAGE_BYTES, sb = sa + A_BYTES;
+            mbar_expect_tx(full_bar + 8 * s, R::STAGE_BYTES);
             tma_load_2d(sa, &mapA, kb * BK, p0, full_bar + 8 * s);
-            tma_load_2d(sb, &mapB, kb * BK, t0, full_bar + 8 * s);
+            tma_load_2d(sb, &mapB, kb * BK, t0 + rank * (BN / CG), full_bar + 8 * s);
             issued = kb + 1;
         }
-    } else if (warp == 1 && lane == 0) {
-        int kb = 0;
-        for (; kb < nk; ++kb) {
+    } else if (warp == 1 && lane == 0 && rank == 1) {
+        // this half of every stage is there: tell rank 0, whose tensor core instructions read both halves
+        const uint32_t remote = map_to_rank(gen_bars + 16 * STAGES, 0);
+        for (int kb = 0; kb < nk; ++kb) {
             const int s = kb % STAGES;
             if (!mbar_wait(full_bar + 8 * s, (uint32_t)((kb / STAGES) & 1)) || *flag) {
                 *flag = 1;
                 break;
             }
+            asm volatile(
+                "fence.release.sync_restrict::shared::cta.cluster;\n"
+                "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote + 8 * s)
+                : "memory");
+        }
+    } else if (warp == 1 && lane == 0) {
+        for (int kb = 0; kb < nk; ++kb) {
+            const int s = kb % STAGES;
+            const uint32_t par = (uint32_t)((kb / STAGES) & 1);
+            if (!mbar_wait(full_bar + 8 * s, par) || (CG == 2 && !mbar_wait(peer_bar + 8 * s, par)) || *flag) {
+                *flag = 1;
+                break;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t sa = sbase + s * STAGE_BYTES, sb = sa + A_BYTES;
+            const uint32_t sa = sbase + s * R::STAGE_BYTES, sb = sa + A_BYTES;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
                 const uint64_t ad = smem_desc_sw128(sa + kk * 32), bd = smem_desc_sw128(sb + kk * 32);
                 const uint32_t acc = (kb > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(kIdesc), "r"(acc));
+                if constexpr (CG == 1)
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                        "l"(ad), "l"(bd), "r"(kIdesc<CG>), "r"(acc));
+                else
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                        "l"(ad), "l"(bd), "r"(kIdesc<CG>), "r"(acc));
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                empty_bar + 8 * s));
+            commit<CG>(empty_bar + 8 * s);
         }
         // the done barrier fires when every MMA issued above has completed
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done_bar));
+        commit<CG>(done_bar);
     }
     __syncwarp();
     bool ok = mbar_wait(done_bar, 0u);
@@ -175,7 +232,9 @@ k_screen_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (good) {
-        const int row = warp * 32 + lane, p = p0 + row;
+        // 32 columns at a time through shared memory (the stages are consumed), so that a
+        // warp stores 128 bytes of one row: a lane per row would touch 32 rows per store
+        float *sh = reinterpret_cast<float *>(gen_base) + warp * 32 * 33;
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 32) {
             uint32_t v[32];
@@ -191,17 +250,27 @@ k_screen_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                   "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (p < P) {
-                float *dst = S + (size_t)p * T + t0 + c0;
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (t0 + c0 + j < T) dst[j] = __uint_as_float(v[j]);
+            for (int j = 0; j < 32; ++j) sh[lane * 33 + j] = __uint_as_float(v[j]);
+            __syncwarp();
+            const int t = t0 + c0 + lane, rows = min(32, P - p0 - warp * 32);
+            if (t < T) {
+                float *dst = S + (size_t)(p0 + warp * 32) * T + t;
+#pragma unroll 8
+                for (int r = 0; r < rows; ++r) dst[(size_t)r * T] = sh[r * 33 + lane];
             }
+            __syncwarp();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+    if constexpr (CG == 1) {
+        if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+    } else {
+        cluster_arrive();   // neither CTA frees its memory while the other may still use it
+        cluster_wait();
+        if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -375,13 +444,24 @@ cudaError_t launch_screen_tc(const void *A, int P, const void *B, int T, int K, 
     // TMA: 16-byte aligned bases and row strides; K a multiple of the 64-element slice
     if (K % BK || (reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(B) & 15))
         return cudaErrorInvalidValue;
-    CUtensorMap ma, mb;
-    if (!make_map(&ma, A, P, K, BM) || !make_map(&mb, B, T, K, BN)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_screen_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    // Two CTAs per tile where every CTA has patterns (an even number of 128-pattern
+    // tiles), the tiles fill the SMs more than once and K is long.  One CTA against two,
+    // K = 4,096, 20,000 templates: 256 patterns 68 -> 66 us, 1,200 (10,000 templates) 94
+    // -> 88; but 128 patterns 41 -> 64, 1,400 (11 tiles) 181 -> 194, 256 x 3,000 27 -> 31
+    // (the pair starts later).  K = 16,384, 2,000 x 39,784: 1.65 -> 1.50 ms.
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const long tiles = (long)((P + BM - 1) / BM) * ((T + BN - 1) / BN);
+    const long num_m = (P + BM - 1) / BM, tiles = num_m * ((T + BN - 1) / BN);
+    const bool pair = num_m % 2 == 0 && tiles > sms && K >= 4096;
+    CUtensorMap ma, mb;
+    if (!make_map(&ma, A, P, K, BM) || !make_map(&mb, B, T, K, pair ? BN / 2 : BN)) return cudaErrorInvalidValue;
     if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
-    k_screen_tc<<<(unsigned)tiles, NT, SMEM_BYTES, st>>>(ma, mb, P, T, K, S, err);
+    if (pair) return launch_clusters(k_screen_tc<2>, 2, NT, Ring<2>::SMEM, tiles / 2, st, ma, mb, P, T, K, S, err);
+    e = cudaFuncSetAttribute(k_screen_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Ring<1>::SMEM);
+    if (e != cudaSuccess) return e;
+    k_screen_tc<1><<<(unsigned)tiles, NT, Ring<1>::SMEM, st>>>(ma, mb, P, T, K, S, err);
     return cudaGetLastError();
 }
 
