@@ -170,6 +170,12 @@ int ndp_operands(xcf_ctx *ctx, const float *img, int P, long img_stride, int row
                  float *out32, void *out16, int *degen, cudaStream_t st) {
     if (n & (n - 1)) return fail(ctx, XCF_ERR_UNIMPLEMENTED, "the NDP needs a 2^k detector side");
     const float sg = ndp_sigma(ctx->opt, n);
+    if (bg_norm_fused(n, sg)) {
+        XCF_LAUNCH(XCF_STAGE_PREP, st,
+                   launch_bg_norm(img, P, img_stride, row_stride, ox, oy, n, sg, out32, out16, degen, st),
+                   "ndp background and normalise");
+        return XCF_OK;
+    }
     if (sg > 0.f) {
         float *tmp, *cor;
         int rc;

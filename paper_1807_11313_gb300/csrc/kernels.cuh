@@ -183,6 +183,11 @@ cudaError_t launch_ndp_norm(const float *img, int P, long img_stride, int row_st
 // blur (sigma px, 0 < sigma <= n), tmp [P][n][n] work array
 cudaError_t launch_ndp_background(const float *img, int P, long img_stride, int row_stride, int ox, int oy, int n,
                                   float sigma, float *tmp, float *out, cudaStream_t st);
+// the same and the contrast normalisation in one kernel: 2^k sides up to 128 at a
+// blur radius of 3 n / 8 (bg_norm_fused)
+bool bg_norm_fused(int n, float sigma);
+cudaError_t launch_bg_norm(const float *img, int P, long img_stride, int row_stride, int ox, int oy, int n, float sigma,
+                           float *out32, void *out16, int *degen, cudaStream_t st);
 // FP32 NDP of pattern p (pn [P][d]) against its candidates cand [P][k] of
 // tn [T][d] (< 0 skipped): best [P] (-1 if degenerate), score [P]
 cudaError_t launch_ndp_rescore(const float *pn, const float *tn, long d, const int *cand, int k, const int *degen,
