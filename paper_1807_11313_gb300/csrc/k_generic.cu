@@ -1,7 +1,7 @@
-// Pre-processing (N in {16, 32, 64, 96, 160}; 128 in k_prep128.cu), the
-// all-sides search kernel for N in {16, 32, 64, 96, 128, 160} and the
-// single-surface peak kernel (128 in k_peak128.cu).  The search and peak kernels
-// hold one N x N complex array in shared memory (rows padded to N + 1) and
+// Pre-processing (N in {16, 32, 64, 96, 160}; 128 in k_prep128.cu), the search
+// kernels for N in {16, 32, 64, 96} (64 and 96: rounds.cuh) and the
+// single-surface peak kernel (128 in k_peak128.cu).  The search at 16 and 32 and
+// the peak kernel hold one N x N complex array in shared memory (rows padded to N + 1) and
 // transform its lines with the warp line FFT (registers and shuffles for
 // N = R x 32 >= 64, mixed radix at 96 and 160; radix-2 butterflies spread
 // over the lanes below 64); the pre-processing transforms two real images per
@@ -44,8 +44,6 @@ constexpr size_t smem_prep_real() {
 // global-load latency of the line transforms
 template <int N>
 constexpr int peak_threads() { return N > 128 ? 1024 : kThreads; }
-template <int N>
-__host__ __device__ constexpr int search_threads() { return N >= 128 ? 1024 : kThreads; }
 
 // PROJ: the image is projected from the master pattern (ps) while it is
 // loaded, instead of read from img (QUAD: from the master's 2 x 2 cells)
@@ -427,7 +425,7 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
 }
 
 template <int N>
-__global__ void __launch_bounds__(search_threads<N>()) k_search_generic(const float2 *__restrict__ St, int T,
+__global__ void __launch_bounds__(kThreads) k_search_generic(const float2 *__restrict__ St, int T,
                                                              const float2 *__restrict__ Sp,
                                                              const int *__restrict__ degen,
                                                              int pairs_per_cta,
@@ -438,7 +436,7 @@ __global__ void __launch_bounds__(search_threads<N>()) k_search_generic(const fl
     if (degen[p]) return;
     const int npairs = ((cand ? kc : T) + 1) / 2;
     const int pb = blockIdx.x * pairs_per_cta, pe = min(npairs, pb + pairs_per_cta);
-    search_body<N, (search_threads<N>() <= 512)>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
+    search_body<N, true>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
 }
 
 // N = 64 and 96: three register rounds on units of 64 and 192 threads: at 64 two
@@ -642,7 +640,7 @@ cudaError_t search_n(const float2 *St, int T, const float2 *Sp, const int *degen
     int ppc = (npairs + chunks - 1) / chunks;
     chunks = (npairs + ppc - 1) / ppc;
     dim3 grid(chunks, P);
-    k_search_generic<N><<<grid, search_threads<N>(), sm, st>>>(St, T, Sp, degen, ppc, keys, peaks_all, cand, kc);
+    k_search_generic<N><<<grid, kThreads, sm, st>>>(St, T, Sp, degen, ppc, keys, peaks_all, cand, kc);
     return cudaGetLastError();
     }
 }
@@ -661,6 +659,8 @@ cudaError_t pair_peak_n(const float2 *St, const int *tidx, const float2 *Sp, con
 
 cudaError_t launch_search128(const float2 *St, int T, const float2 *Sp, const int *degen, int P,
                              unsigned long long *keys, float *peaks_all, int num_sms, cudaStream_t st);
+cudaError_t launch_search128_list(const float2 *St, const int *cand, int kc, const float2 *Sp, const int *degen, int P,
+                                  unsigned long long *keys, int num_sms, cudaStream_t st);
 
 cudaError_t launch_prep(const float *img, int P, const PrepArgs &a, float2 *spec, float *spatial,
                         int *degen, const int *active, cudaStream_t st) {
@@ -708,12 +708,6 @@ cudaError_t launch_search(int N, const float2 *St, int T, const float2 *Sp, cons
     }
 }
 
-cudaError_t launch_search_generic128(const float2 *St, int T, const float2 *Sp, const int *degen, int P,
-                                     unsigned long long *keys, float *peaks_all, int num_sms,
-                                     cudaStream_t st) {
-    return search_n<128>(St, T, Sp, degen, P, keys, peaks_all, num_sms, st);
-}
-
 cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc, const float2 *Sp,
                                const int *degen, int P, unsigned long long *keys, float *peaks, int num_sms,
                                cudaStream_t st) {
@@ -722,7 +716,8 @@ cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc,
         case 16: return search_n<16>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         case 32: return search_n<32>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         case 64: return search_n<64>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
-        case 128: return search_n<128>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
+        case 128:   // St: the search layout, as for the search itself
+            return peaks ? cudaErrorInvalidValue : launch_search128_list(St, cand, kc, Sp, degen, P, keys, num_sms, st);
         case 96: return search_n<96>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
         case 160:
         case 200: return launch_search_lines(N, St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);

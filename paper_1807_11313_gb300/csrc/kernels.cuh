@@ -66,7 +66,8 @@ cudaError_t launch_pair_peak_c256(const float2 *St, const int *tidx, const float
 cudaError_t launch_prep_c256(const float *img, int P, const PrepArgs &a, float2 *spec, float *spatial, int *degen,
                              const int *active, cudaStream_t st);
 
-// search over each pattern's candidate list cand [P][kc] (library indices, < 0 empty)
+// search over each pattern's candidate list cand [P][kc] (library indices, < 0 empty);
+// N = 128: St in the search layout, no peaks
 cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc, const float2 *Sp,
                                const int *degen, int P, unsigned long long *keys, float *peaks, int num_sms,
                                cudaStream_t st);

@@ -84,11 +84,13 @@ __device__ __forceinline__ float fft32_rest_max(float2 (&x)[32]) {
 // by group 1).  Runs on the calling CTA's NT threads and SMEM_BYTES of dynamic
 // shared memory (named barriers 1 and 2) and folds the best (peak, template)
 // of the item into keys[p].  ALL: also write every template's peak to
-// peaks_all [P][T].
-template <bool ALL>
+// peaks_all [P][T].  LIST: the T positions are the pattern's candidate list
+// (library indices in any order, < 0: none).
+template <bool ALL, bool LIST = false>
 __device__ __forceinline__ void search_body(const float2 *__restrict__ Spk, int T, const float2 *__restrict__ Sp,
                                               int p, int pb, int pe, unsigned long long *__restrict__ keys,
-                                              float *__restrict__ peaks_all) {
+                                              float *__restrict__ peaks_all, const int *__restrict__ list = nullptr) {
+    static_assert(!(ALL && LIST), "lists keep the best only");
     using namespace fft128;
     extern __shared__ float4 smem_raw[];
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
@@ -106,6 +108,14 @@ __device__ __forceinline__ void search_body(const float2 *__restrict__ Spk, int 
     const bool special = g == 0;
     float2 *own = buf + warp * 1024;   // this warp's region
 
+    const int te = min(2 * pe, T);
+    auto id = [&](int j) { return LIST ? __ldg(list + j) : j; };
+    // the group's next position from j on with a template (te or above: none)
+    auto used = [&](int j) {
+        if (LIST)
+            while (j < te && id(j) < 0) j += 2;
+        return j;
+    };
     // a template's columns 0..63 fill the group's buffer exactly; each warp copies into its region
     auto stage = [&](int t) {
         const float4 *s = reinterpret_cast<const float4 *>(Spk + (size_t)t * SPEC);
@@ -143,23 +153,23 @@ __device__ __forceinline__ void search_body(const float2 *__restrict__ Spk, int 
         else if (threadIdx.x < 256)
             tw2[threadIdx.x - 128] = w128((threadIdx.x & 31) * ((threadIdx.x - 128) >> 5));   // [k3][g]
     }
-    const int te = min(2 * pe, T);
-    int t = 2 * pb + grp;
+    int t = used(2 * pb + grp);
     if (t < te) {
-        stage_edge(t);
-        stage(t);
+        stage_edge(id(t));
+        stage(id(t));
         cp_async_wait_all();
     }
     __syncthreads();   // the pattern and the tables are in place
     if (t < te) make_p0();
 
-    float best_v = -INFINITY;   // this thread's largest value and its template (ascending: the lowest among equals)
+    float best_v = -INFINITY;   // this thread's largest value and its template (the lowest among equals)
     int best_t = -1;
 
     // Per template three barriers of the group: the staged template is complete; it
     // has been read (the register work of round 1 runs before this one); the columns
     // are exchanged.  From there on a warp works in its own region alone.
-    for (int it = 0; t < te; t += 2, ++it) {
+    for (int it = 0, tn; t < te; t = tn, ++it) {
+        tn = used(t + 2);
         cp_async_wait_all();
         sync();   // buf holds template t, p0 its packed column; the previous round 3 is done with buf
         if (ALL && it > 0 && tid == 0) {
@@ -214,7 +224,7 @@ __device__ __forceinline__ void search_body(const float2 *__restrict__ Spk, int 
             for (int l = 0; l < 8; ++l) x[k][l] = src[l * 128];
         }
         __syncwarp();   // the warp has read its columns: its region is free
-        if (t + 2 < te) stage_edge(t + 2);   // edge was last read for this template's p0
+        if (tn < te) stage_edge(id(tn));   // edge was last read for this template's p0
 #pragma unroll
         for (int k = 0; k < 4; ++k) fft_reg_dif<8, +1>(x[k]);   // x[k][bitrev(j)] = row k2 + 16 j
         {
@@ -255,19 +265,19 @@ __device__ __forceinline__ void search_body(const float2 *__restrict__ Spk, int 
             }
         }
         __syncwarp();   // every lane holds its line's values: the region is free
-        if (t + 2 < te) stage(t + 2);
+        if (tn < te) stage(id(tn));
         dif_stage<32, 0>(z);
         float m = fft32_rest_max(z);
-        if (m > best_v) {
+        if (m > best_v || (LIST && m == best_v && id(t) < best_t)) {
             best_v = m;
-            best_t = t;
+            best_t = id(t);
         }
         if (ALL) {
 #pragma unroll
             for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
             if (lane == 0) reinterpret_cast<float *>(sm + OFF_RED + grp * 8)[(it & 1) * 8 + warp] = m;
         }
-        if (t + 2 < te) {   // the next template's edge columns (all but the newest copy group have landed)
+        if (tn < te) {   // the next template's edge columns (all but the newest copy group have landed)
             cp_async_wait_one();
             make_p0();
         }

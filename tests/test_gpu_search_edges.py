@@ -99,7 +99,7 @@ def test_search_64_and_96(px, n, T, P):
     check_search(px, n, T, P, native=1)
 
 
-@pytest.mark.parametrize("n", [64, 96, 160, 200, 256])
+@pytest.mark.parametrize("n", [64, 96, 128, 160, 200, 256])
 @pytest.mark.parametrize("k", [1, 2, 5, 8])
 def test_candidate_lists(px, n, k):
     """Lists with empty entries, repeated templates (ties to the lowest index)
@@ -142,3 +142,26 @@ def test_search_160_and_200(px, n, T, P):
 @pytest.mark.parametrize("P", [1, 3, 80])
 def test_search_256(px, T, P):
     check_search(px, 256, T, P)
+
+
+def test_long_candidate_lists_128(px):
+    """Lists in several parts, with runs of empty entries longer than a part's step."""
+    n, T, P, k = 128, 70, 4, 64
+    ctx = px.Context()
+    g = px.geometry(n, n)
+    q = torch.zeros((T, 4), dtype=torch.float64, device="cuda")
+    q[:, 0] = 1
+    lib = px.xcf_build_library_images(ctx, _images(n, T, 8), q, g)
+    pats = _images(n, P, 9)
+    cand = torch.stack([torch.randperm(T, generator=torch.Generator().manual_seed(p))[:k] for p in range(P)]).int()
+    cand[1, 5:40] = -1
+    cand[2, :63] = -1
+    cand[3, 1::2] = -1
+    best, peak, _ = px.xcf_rescore(ctx, lib, pats, cand.cuda())
+    ref = _reference(lib.spectra(), px.xcf_prep(ctx, pats, g)[0])
+    for p in range(P):
+        c = cand[p][cand[p] >= 0].cuda().long()
+        assert int(best[p]) == int(c[ref[p, c].argmax()])
+        torch.testing.assert_close(peak[p].double(), ref[p, c].amax(), rtol=1e-4, atol=1e-6)
+    lib.close()
+    ctx.close()
