@@ -23,15 +23,17 @@
 // What bounds it: sixteen warps go through the passes together, and the load
 // queue (64 global and 16 cluster loads per thread and template) fills in the
 // first and third; issue is active 42 %.  300 patterns x 1,018 templates: 53.6 ->
-// 39.7 ms (15.9 -> 22 TFLOP/s, 27 % of the FP32 peak) against template pairs on
-// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.64 ms.  A
-// full release at the barrier between the column and line passes costs 3 % of that
-// (40.8, 4.76).
+// 38.9 ms (15.9 -> 22.1 TFLOP/s, 27 % of the FP32 peak) against template pairs on
+// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.49 ms.  A
+// full release at the barrier between the column and line passes costs 3 % of that.
 // Measured without gain: 16-byte template loads from an aligned copy of the
 // library with half of the pattern in shared memory (41.3), the next template's
 // first values loaded a pass ahead (49.4: spills), 1,024 threads at 64 registers
-// (42.2), all gathers as cluster loads (41.6).  The templates stay in the plain
+// (42.2), all gathers as cluster loads (41.6); two clusters of four CTAs per four SMs
+// (passes256.cuh) 40.3, the rescore 4.42.  The templates stay in the plain
 // layout: no second copy of the library (5.5 GB at 20,000 templates).
+#include <algorithm>
+
 #include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
@@ -93,7 +95,7 @@ __device__ __forceinline__ void gather(float2 (&z)[2][16], const float2 *buf, ui
 template <bool ALL>
 __global__ void __launch_bounds__(NT, 1)
 k_search256(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, const int *__restrict__ degen,
-            int nchunks, int per, int n_items, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
+            int P, int per, int n_items, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
             const int *__restrict__ cand, int kc) {
     extern __shared__ float4 smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
@@ -124,7 +126,8 @@ k_search256(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp,
         }
     };
     for (int item = cid; item < n_items; item += ncl) {
-        const int p = item / nchunks, jb = (item - p * nchunks) * per, je = min(n, jb + per);
+        // part by part: the clusters that run together read the same templates
+        const int part = item / P, p = item - part * P, jb = part * per, je = min(n, jb + per);
         if (degen[p]) continue;   // uniform over the cluster, as every bound below
         const float2 *sp = Sp + (size_t)p * N * HW;
         float2 s0 = make_float2(0.f, 0.f), sh = s0;   // the pattern's columns 0 and 128 at row tid
@@ -289,14 +292,29 @@ cudaError_t launch_search_c256(const float2 *St, int T, const float2 *Sp, const 
     int ncl_max = 0;
     const cudaError_t e = resident_clusters(kern, NC, NT, sizeof(Smem), resident[peaks_all ? 1 : 0], &ncl_max);
     if (e != cudaSuccess) return e;
-    // chunks of templates so that there are at least ~4 items per resident cluster
-    const long want = 4L * ncl_max;
-    int nchunks = (int)((want + P - 1) / P);
-    nchunks = nchunks < 1 ? 1 : (nchunks > n ? n : nchunks);
+    // each pattern's templates in c parts, c minimising rounds of items over the resident
+    // clusters x time of an item (a part starts with the pattern's columns 0 and 128 and
+    // ends with a reduction: half a template's time).  Items go part by part: pattern by
+    // pattern, the running clusters spread over the library and miss L2 (300 x 1,018:
+    // 40.2 ms, part by part 38.9, whole items 39.7).  Against about four items per cluster
+    // whatever the remainder, 2,000 templates: 10 patterns 3.25 -> 2.61 ms, 77: 24.6 ->
+    // 19.9, 500: 136 -> 128; 32 candidates of 77 patterns 432 -> 402 us, of 1,000 4.65 ->
+    // 4.49 ms.
+    int nchunks = 1;
+    long least = -1;
+    const int most = (int)std::min<long>(n, std::max<long>(64, 4L * ncl_max / P));
+    for (int c = 1; c <= most; ++c) {
+        const int len = (n + c - 1) / c;
+        const long rounds = ((long)P * ((n + len - 1) / len) + ncl_max - 1) / ncl_max, cost = rounds * (2L * len + 1);
+        if (least < 0 || cost <= least) {
+            least = cost;
+            nchunks = c;
+        }
+    }
     const int per = (n + nchunks - 1) / nchunks;
     nchunks = (n + per - 1) / per;
     const long n_items = (long)P * nchunks;
     if (n_items > (1L << 30)) return cudaErrorInvalidValue;
     return launch_clusters(kern, NC, NT, sizeof(Smem), n_items < ncl_max ? n_items : ncl_max, st, St, T, Sp, degen,
-                           nchunks, per, (int)n_items, keys, peaks_all, cand, kc);
+                           P, per, (int)n_items, keys, peaks_all, cand, kc);
 }
