@@ -190,7 +190,7 @@ def _roofline_traffic(meta_name: str, sources):
     return m.get("bytes_per_launch_full")
 
 
-SEARCH128_SOURCES = ("search128.cuh", "k_search128.cu")
+SEARCH128_SOURCES = ("fft128.cuh", "search128.cuh", "k_search128.cu")
 
 
 def _l2_note(pattern_bytes, lib_bytes, what):
@@ -369,7 +369,7 @@ def run_precision(args, px, torch, dev, rank, world, local, dist, emit=True):
                    "frac": achieved / tensor_peak, "traffic": None, "kernel": "k_screen_tc",
                    "peak_basis": "measured sustained cuBLAS BF16 (MEASURED_PEAKS.json)" if pk else "fallback",
                    "screen_ms_per_launch": s_ms / max(s_n, 1), "launches_per_step": s_n / args.steps}
-    # the dominant stage: the FP32 FFT rescore of the k candidates (k_search_c256, candidate-list mode)
+    # the dominant stage: the FP32 FFT rescore of the k candidates (k_search256, candidate-list mode)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     sm_max = pk.get("sm_max_mhz") or (clocks or {}).get("sm_max_mhz") or 2070.0
     fp32_peak = sms * 128 * 2 * sm_max * 1e6 / 1e12
@@ -377,7 +377,7 @@ def run_precision(args, px, torch, dev, rank, world, local, dist, emit=True):
     r_ach = P * k * flops_per_pair(n) / (r_ms / 1e3) / 1e12
     stages = {kk: v[0] / args.steps for kk, v in prof.items()}
     roofline = {"bound": "alu", "achieved": r_ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": r_ach / fp32_peak,
-                "traffic": None, "kernel": "k_search_c256w (rescore of the top-k candidates)",
+                "traffic": None, "kernel": "k_search256 (rescore of the top-k candidates)",
                 "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz",
                 "stage_share": r_ms / max(sum(stages.values()), 1e-9),
                 "stage_ms_per_step": stages, "secondary": {"screen": screen_roof}}
@@ -630,7 +630,7 @@ def run_net(args, px, torch, dev, rank, world, local, dist):
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         sm_max = (pk or {}).get("sm_max_mhz") or (clocks or {}).get("sm_max_mhz") or 2070.0
         peak, bound, basis = sms * 128 * 2 * sm_max * 1e6 / 1e12, "alu", "152 SMs x 128 FP32 lanes x 2 x clock"
-        kern = "proposal network forward (k_gemm, FP32)"
+        kern = "proposal network forward (k_conv32, FP32)"
     else:
         peak, bound = (pk or {}).get("bf16_tflops_sustained") or 1700.0, "tensor"
         basis = "measured sustained cuBLAS BF16 (MEASURED_PEAKS.json)" if pk else "fallback"
@@ -850,9 +850,9 @@ def run_batched(args, px, torch, dev, rank, world, local, dist, emit=True):
         d["frac"] = d["achieved_tflops"] / fp32_peak
     achieved = flops / (search_ms_call / 1e3) / 1e12
     kernels = {16: "k_search_maps", 32: "k_search_maps", 64: "k_search_maps", 96: "k_search_maps",
-               128: "k_search_maps", 160: "k_search_maps", 200: "k_search_n200", 256: "k_search_c256w"}
+               128: "k_search_maps", 160: "k_search_maps", 200: "k_search_lines", 256: "k_search256"}
     body_names = {0: "warp lines (R x 32)", 1: "three rounds (16x8 | 4x32)", 2: "radix-2 in shared memory",
-                  3: "eight-lane groups (8 x 8)"}
+                  3: "register rounds on 64-thread units"}
     tuning = {}
     for (lib, _), n in zip(batch, ns):
         t = px.xcf_maps_get_tuning(ctx, n, lib.T)
@@ -1081,7 +1081,7 @@ def run_learned(args, px, torch, dev, rank, world, local, dist, emit=True):
     net_ms, net_n = prof["net"]
     net_flops = CNN_FORWARD_FLOPS * n_test * args.steps
     if args.net_fp32:
-        net_peak, bound, kern, basis = fp32_peak, "alu", "proposal network forward (k_gemm, FP32)", "FP32 ALU"
+        net_peak, bound, kern, basis = fp32_peak, "alu", "proposal network forward (k_conv32, FP32)", "FP32 ALU"
     else:
         net_peak = (pk or {}).get("bf16_tflops_sustained") or 1700.0
         bound, kern = "tensor", "proposal network forward (convolution 1 direct FP32 -> BF16; 2-5 k_conv_tc implicit GEMM, tcgen05 BF16)"
@@ -1091,7 +1091,7 @@ def run_learned(args, px, torch, dev, rank, world, local, dist, emit=True):
                 "stage_ms_per_step": {kk: v[0] / args.steps for kk, v in prof.items()}}
     roofline["frac"] = roofline["achieved"] / net_peak if roofline["achieved"] else None
     net_roof = roofline
-    # the dominant stage: pre-processing (k_prep_real).  Timed alone on the step's own test patterns (spectra
+    # the dominant stage: pre-processing (k_prep128).  Timed alone on the step's own test patterns (spectra
     # and filtered images, as the learned path takes them); algorithmic bytes: the image in, the half spectrum
     # and the filtered image out
     stages = {kk: v[0] / args.steps for kk, v in prof.items()}
@@ -1106,7 +1106,7 @@ def run_learned(args, px, torch, dev, rank, world, local, dist, emit=True):
     prep_bytes = n_test * (4 * n * n + 8 * n * (n // 2 + 1) + 4 * n * n)
     hbm = (pk or {}).get("hbm_gbs") or 6800.0
     roofline = {"bound": "hbm", "achieved": prep_bytes / (prep_ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
-                "traffic": None, "kernel": "k_prep_real (pre-processing: crop, statistics, window, FFT, band-pass, "
+                "traffic": None, "kernel": "k_prep128 (pre-processing: crop, statistics, window, FFT, band-pass, "
                 "norm, filtered image)", "peak_basis": "measured copy bandwidth (MEASURED_PEAKS.json)" if pk else
                 "fallback", "timed": f"alone on the {n_test} test patterns, {prep_ms:.2f} ms per launch",
                 "stage_share": stages.get("prep", 0.0) / max(sum(stages.values()), 1e-9),
