@@ -173,6 +173,13 @@ k_screen_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             tma_load_2d(sb, &mapB, kb * BK, t0 + rank * (BN / CG), full_bar + 8 * s);
             issued = kb + 1;
         }
+        // rank 0's commits arrive on this CTA's barriers: they have before it leaves
+        if (CG == 2)
+            for (int kb = max(0, nk - STAGES); kb < issued && issued == nk; ++kb)
+                if (!mbar_wait(empty_bar + 8 * (kb % STAGES), (uint32_t)((kb / STAGES) & 1))) {
+                    *flag = 1;
+                    break;
+                }
     } else if (warp == 1 && lane == 0 && rank == 1) {
         // this half of every stage is there: tell rank 0, whose tensor core instructions read both halves
         const uint32_t remote = map_to_rank(gen_bars + 16 * STAGES, 0);
