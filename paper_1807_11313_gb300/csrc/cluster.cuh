@@ -10,10 +10,13 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// without release: orders reads already consumed before it against writes after the wait
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+// releases every access before it.  The form for a thread that has read another
+// CTA's shared memory, whose owner overwrites it after the wait: only a release
+// orders those loads before the owner's stores
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-// releases this CTA's own shared memory only: does not wait for global stores in flight
+// releases accesses to this CTA's own shared memory only, for values that the others
+// read after the wait: does not wait for global stores in flight, and orders no read of
+// another CTA's shared memory
 __device__ __forceinline__ void cluster_arrive_shared() {
     asm volatile("fence.release.sync_restrict::shared::cta.cluster;\nbarrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }

@@ -101,8 +101,8 @@ k_peak256(const float2 *__restrict__ St, const int *__restrict__ tidx, const flo
         // ---- lines
         float2 z[2][16];
         gather_lines(z, base, OWN * c + lr, b);
-        cluster_arrive_relaxed();   // this thread has gathered (and used) its values
-        cluster_wait();             // every thread of the cluster has: the buffer takes the lines
+        cluster_arrive();   // releases this thread's gathers
+        cluster_wait();     // every thread of the cluster has its values: the buffer takes the lines
         float bv = -INFINITY;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -135,6 +135,7 @@ k_peak256(const float2 *__restrict__ St, const int *__restrict__ tidx, const flo
         if (lane == 0) sm.top[warp] = make_float2(bv, __int_as_float(bi));
         cluster_arrive_shared();
         cluster_wait();   // lines and maxima are in place
+        float c0 = 0.f, cxm = 0.f, cxp = 0.f, cym = 0.f, cyp = 0.f;
         if (c == 0 && warp == 0) {
             const float2 v = ld_cluster(map_to_rank(&sm.top[lane & (NT / 32 - 1)], lane / (NT / 32)));
             bv = v.x;
@@ -149,17 +150,21 @@ k_peak256(const float2 *__restrict__ St, const int *__restrict__ tidx, const flo
             const int x = (x0 + (lane == 1 ? N - 1 : lane == 2 ? 1 : 0)) & (N - 1);
             const float2 w = ld_cluster(map_to_rank(buf + (y & (OWN - 1)) * N + x, (y & 127) / OWN));
             const float mine = y & 128 ? w.y : w.x;
-            const float c0 = __shfl_sync(0xffffffffu, mine, 0), cxm = __shfl_sync(0xffffffffu, mine, 1),
-                        cxp = __shfl_sync(0xffffffffu, mine, 2), cym = __shfl_sync(0xffffffffu, mine, 3),
-                        cyp = __shfl_sync(0xffffffffu, mine, 4);
-            if (lane == 0) {
-                peak[p] = c0;
-                shift[2 * p] = (float)(x0 < N / 2 ? x0 : x0 - N) + parabola_c(cxm, c0, cxp);
-                shift[2 * p + 1] = (float)(y0 < N / 2 ? y0 : y0 - N) + parabola_c(cym, c0, cyp);
-                if (argmax) argmax[p] = bi;
-            }
+            c0 = __shfl_sync(0xffffffffu, mine, 0);
+            cxm = __shfl_sync(0xffffffffu, mine, 1);
+            cxp = __shfl_sync(0xffffffffu, mine, 2);
+            cym = __shfl_sync(0xffffffffu, mine, 3);
+            cyp = __shfl_sync(0xffffffffu, mine, 4);
         }
-        cluster_arrive_relaxed();   // CTA 0 has read the other CTAs' lines and maxima
+        cluster_arrive();   // releases CTA 0's reads of the other CTAs' lines and maxima (the results follow it: no store to wait for)
+        if (c == 0 && tid == 0) {
+            const int y0 = bi >> 8, x0 = bi & (N - 1);
+            peak[p] = c0;
+            shift[2 * p] = (float)(x0 < N / 2 ? x0 : x0 - N) + parabola_c(cxm, c0, cxp);
+            shift[2 * p + 1] = (float)(y0 < N / 2 ? y0 : y0 - N) + parabola_c(cym, c0, cyp);
+            if (argmax) argmax[p] = bi;
+        }
+        __syncwarp();
         cluster_wait();
     }
     cluster_arrive();   // no CTA leaves while another may still read its shared memory

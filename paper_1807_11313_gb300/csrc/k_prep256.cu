@@ -187,8 +187,8 @@ k_prep256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
                 });
                 fft_reg_dif<16, -1>(x[h]);
             }
-            cluster_arrive_relaxed();   // this thread has gathered (and used) its values
-            cluster_wait();             // every thread of the cluster has: the buffer takes the columns
+            cluster_arrive();   // releases this thread's gathers
+            cluster_wait();     // every thread of the cluster has its values: the buffer takes the columns
 #pragma unroll
             for (int h = 0; h < 2; ++h) column_store<-1>(x[h], buf, sm.tw, ql, a8, h);
             __syncthreads();
@@ -243,6 +243,8 @@ k_prep256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
             for (int i = tid; i < 2 * OWN * HW; i += NT) out[(size_t)2 * OWN * c * HW + i] = make_float2(0.f, 0.f);
             if (spatial)
                 for (int i = tid; i < 2 * OWN * N; i += NT) spatial[(size_t)p * N * N + (size_t)2 * OWN * c * N + i] = 0.f;
+            cluster_arrive();   // releases the reads of the warps' sums, as the arrivals after the gathers do otherwise
+            cluster_wait();
             continue;
         }
 #pragma unroll
@@ -281,8 +283,8 @@ k_prep256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__
         cluster_arrive_shared();
         cluster_wait();   // the columns are complete
         gather_lines(z, base, OWN * c + lr, b);
-        cluster_arrive_relaxed();
-        cluster_wait();   // the buffer takes the lines
+        cluster_arrive();   // releases this thread's gathers
+        cluster_wait();     // the buffer takes the lines
         const float inv_n = 1.f / N;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {

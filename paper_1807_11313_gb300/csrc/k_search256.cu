@@ -216,8 +216,8 @@ k_search256(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp,
             else gather<1>(z, buf, base0, base1, OWN * c + lr, b);
 #pragma unroll
             for (int h = 0; h < 2; ++h) fft_reg_dif<16, +1>(z[h]);
-            cluster_arrive_relaxed();   // this thread has gathered (and used) its values
-            cluster_wait();             // every thread of both CTAs has: the buffer takes the lines
+            cluster_arrive();   // releases this thread's gathers
+            cluster_wait();     // every thread of both CTAs has its values: the buffer takes the lines
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float2 *dst = buf + (lr + 32 * h) * 256 + (b & 1);
