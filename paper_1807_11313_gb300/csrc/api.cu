@@ -589,32 +589,50 @@ int xcf_build_library_images(xcf_ctx *ctx, const float *images, const double *qu
 }
 
 namespace {
-// The library's own copies of the orientations and the master, in one
-// allocation with the master's 2 x 2 cells.  The cells are kept for masters up
-// to half the 129 MB L2 (M <= 1,448), where they stay resident beside the
-// spectra; a larger master, or one whose cells find no memory (32 M^2 bytes),
-// is read as it is.
-constexpr size_t kQuadMaxBytes = (size_t)64 << 20;
-cudaError_t library_head(xcf_library *lib, const double *quats, const float *master, cudaStream_t st) {
+// A library's spectra (if it has any), and its own copies of the orientations and the
+// master, with the master's 2 x 2 cells (32 M^2 bytes) at the end of one of the two
+// allocations.
+//
+// cudaMalloc serves a request of up to about 2 MB from a block that it holds and maps
+// memory for a larger one, 140 us with cudaFree.  So the cells join an allocation that is
+// mapped without them, the master's or else the spectra's; a library with neither (a few
+// templates of a master with M < 512) does without.  Against cells beside the master
+// always, M = 256: 10 templates at 64 px 197 -> 56 us, 300 at 128 px 352 -> 301; what the
+// small library loses, 64 patterns refined at 128 px: 180 -> 194 us.  M = 1,024, 10 at 64
+// px: 200 us without cells, 221 with, and the refinement of 4 patterns at 128 px 13 us less.
+// Kept where a lookup may read them (bilinear) from L2 beside the spectra (M <= 1,448, half
+// of the 129 MB); where they find no memory the master is read as it is.
+constexpr size_t kCellsMaxBytes = (size_t)64 << 20, kMappedBytes = (size_t)2 << 20;
+cudaError_t library_memory(const xcf_ctx *ctx, xcf_library *lib, bool spectra, const double *quats,
+                           const float *master, cudaStream_t st) {
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t mm = 2 * (size_t)lib->M * lib->M, qb = up(sizeof(double) * 4 * lib->T);
-    const size_t mb = master ? up(sizeof(float) * mm) : 0;
-    size_t quad = master && sizeof(float4) * mm <= kQuadMaxBytes ? sizeof(float4) * mm : 0;
-    cudaError_t e = cudaMalloc(&lib->head, qb + mb + quad);
-    if (e != cudaSuccess && quad) {
-        cudaGetLastError();
-        quad = 0;
-        e = cudaMalloc(&lib->head, qb + mb);
-    }
+    const size_t mm = 2 * (size_t)lib->M * lib->M, T = lib->T;
+    const size_t sb = spectra ? up(sizeof(float2) * lib->N * (lib->N / 2 + 1) * T) : 0;
+    const size_t qb = up(sizeof(double) * 4 * T), hb = qb + (master ? up(sizeof(float) * mm) : 0);
+    const size_t cells = sizeof(float4) * mm;
+    const bool wanted = master && ctx->opt.master_interp == 0 && cells <= kCellsMaxBytes;
+    char *spec = nullptr, *head = nullptr, *quad = nullptr;
+    auto alloc = [&](char **p, size_t bytes, bool with_cells) {
+        if (with_cells) {
+            if (cudaMalloc(p, bytes + cells) == cudaSuccess) {
+                quad = *p + bytes;
+                return cudaSuccess;
+            }
+            cudaGetLastError();
+        }
+        return cudaMalloc(p, bytes);
+    };
+    cudaError_t e = sb ? alloc(&spec, sb, wanted && hb <= kMappedBytes && sb > kMappedBytes) : cudaSuccess;
+    lib->spectra = reinterpret_cast<float2 *>(spec);
+    if (e == cudaSuccess) e = alloc(&head, hb, wanted && hb > kMappedBytes);
     if (e != cudaSuccess) return e;
-    char *base = static_cast<char *>(lib->head);
-    lib->quats = reinterpret_cast<double *>(base);
-    e = cudaMemcpyAsync(lib->quats, quats, sizeof(double) * 4 * lib->T, cudaMemcpyDeviceToDevice, st);
+    lib->quats = reinterpret_cast<double *>(head);
+    e = cudaMemcpyAsync(lib->quats, quats, sizeof(double) * 4 * T, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess || !master) return e;
-    lib->master = reinterpret_cast<float *>(base + qb);
+    lib->master = reinterpret_cast<float *>(head + qb);
     e = cudaMemcpyAsync(lib->master, master, sizeof(float) * mm, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess || !quad) return e;
-    lib->quad = reinterpret_cast<float4 *>(base + qb + mb);
+    lib->quad = reinterpret_cast<float4 *>(quad);
     return launch_master_quads(lib->master, lib->M, lib->quad, st);
 }
 
@@ -644,9 +662,8 @@ int build_from_master(xcf_ctx *ctx, const float *master, int32_t M, const double
     lib->oy = c.oy;
     memcpy(lib->pc, c.pc, sizeof c.pc);
     const size_t H = (size_t)c.n * (c.n / 2 + 1);
-    cudaError_t e = spectra ? cudaMalloc(&lib->spectra, sizeof(float2) * H * T) : cudaSuccess;
-    if (e == cudaSuccess) e = library_head(lib, quats, master, st);
-    if (!lib->head) {
+    cudaError_t e = library_memory(ctx, lib, spectra, quats, master, st);
+    if (!lib->quats) {
         cudaGetLastError();
         xcf_library_free(lib);
         return fail(ctx, XCF_ERR_OOM, "xcf_build_library: allocation failed");
@@ -715,9 +732,8 @@ int build_from_images(xcf_ctx *ctx, const float *images, const double *quats, in
     lib->oy = c.oy;
     memcpy(lib->pc, c.pc, sizeof c.pc);
     const size_t H = (size_t)c.n * (c.n / 2 + 1);
-    cudaError_t e = spectra ? cudaMalloc(&lib->spectra, sizeof(float2) * H * T) : cudaSuccess;
-    if (e == cudaSuccess) e = library_head(lib, quats, master, st);
-    if (!lib->head) {
+    cudaError_t e = library_memory(ctx, lib, spectra, quats, master, st);
+    if (!lib->quats) {
         cudaGetLastError();
         xcf_library_free(lib);
         return fail(ctx, XCF_ERR_OOM, "xcf_build_library_images: allocation failed");
@@ -754,7 +770,7 @@ int xcf_library_free(xcf_library *lib) {
     if (lib->spectra_pk) cudaFree(lib->spectra_pk);
     if (lib->bf16) cudaFree(lib->bf16);
     if (lib->ndp32) cudaFree(lib->ndp32);
-    if (lib->head) cudaFree(lib->head);
+    if (lib->quats) cudaFree(lib->quats);
     delete lib;
     return XCF_OK;
 }

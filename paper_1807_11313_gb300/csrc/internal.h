@@ -117,10 +117,10 @@ struct xcf_library {
     void *bf16 = nullptr;           // screen: unit-norm filtered images [T][N*N] in BF16
     float *ndp32 = nullptr;         // NDP: contrast-normalised images / N [T][N*N] in FP32 ...
     void *ndp16 = nullptr;          // ... and in BF16 (inside the same allocation)
-    double *quats = nullptr;        // [T][4] ...
-    float *master = nullptr;        // ... the master [2][M][M] (null without one) ...
-    float4 *quad = nullptr;         // ... and the master as 2 x 2 cells (null: lookups read the master itself)
-    void *head = nullptr;           // the one allocation that holds these three
+    double *quats = nullptr;        // [T][4], and in the same allocation ...
+    float *master = nullptr;        // ... the master [2][M][M] (null without one)
+    float4 *quad = nullptr;         // the master as 2 x 2 cells, behind the spectra or the master (null: lookups
+                                    // read the master itself)
 };
 
 // the side whose search kernel reads the templates in a layout of its own (as
