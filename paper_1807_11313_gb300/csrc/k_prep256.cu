@@ -57,14 +57,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// 1 / sqrt(v), v > 0: one Newton step in FP64 on the FP32 value (every warp of the
-// CTA waits for it: a third of the FP64 square root and division's latency)
-__device__ __forceinline__ float inv_sqrt(double v) {
-    if (!(v > 1e-30 && v < 1e30)) return (float)(1.0 / sqrt(v));
-    const double r = (double)rsqrtf((float)v);
-    return (float)(r * (1.5 - 0.5 * v * r * r));
-}
-
 __global__ void __launch_bounds__(NT, 2)
 k_prep256(const float *__restrict__ img, int P, PrepArgs a, float2 *__restrict__ spec, float *__restrict__ spatial,
           int *__restrict__ degen, const int *__restrict__ active) {
