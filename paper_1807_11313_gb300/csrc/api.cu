@@ -1276,7 +1276,7 @@ int xcf_rescore(xcf_ctx *ctx, const xcf_library *lib, const float *patterns, int
         XCF_CHECK(cudaMemsetAsync(keys, 0, sizeof(unsigned long long) * np, st), "memset keys");
         if (c.n != 256) {
             XCF_LAUNCH(XCF_STAGE_SEARCH, st,
-                       launch_search_list(c.n, search_spectra(lib), cp, k, sp, degen, np, keys, nullptr, ctx->num_sms, st),
+                       launch_search_list(c.n, search_spectra(lib), cp, k, sp, degen, np, keys, ctx->num_sms, st),
                        "rescore");
         } else {
             XCF_LAUNCH(XCF_STAGE_SEARCH, st,
@@ -1339,8 +1339,7 @@ int xcf_index_precision(xcf_ctx *ctx, const xcf_library *lib, const float *patte
         XCF_CHECK(cudaMemsetAsync(keys, 0, sizeof(unsigned long long) * np, st), "memset keys");
         if (c.n != 256) {
             XCF_LAUNCH(XCF_STAGE_SEARCH, st,
-                       launch_search_list(c.n, search_spectra(lib), cand, k, spec, degen, np, keys, nullptr, ctx->num_sms,
-                                          st),
+                       launch_search_list(c.n, search_spectra(lib), cand, k, spec, degen, np, keys, ctx->num_sms, st),
                        "rescore");
         } else {
             XCF_LAUNCH(XCF_STAGE_SEARCH, st,

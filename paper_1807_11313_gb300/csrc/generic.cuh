@@ -174,7 +174,6 @@ __device__ inline float block_max(float v, float *sh, const Grp &g) {
     g.sync();
     return r;
 }
-__device__ inline float block_max(float v, float *sh) { return block_max(v, sh, cta_group()); }
 
 // Z = X1 + i X2 over the full N x N spectrum, X_j = conj(St_j) Sp extended
 // from the stored half (columns 0..N/2) by Hermitian symmetry.
@@ -226,26 +225,19 @@ __device__ __forceinline__ void pair_row_make(float2 (&v)[N / 32], const PairRow
         v[j] = c <= N / 2 ? make_float2(x1.x - x2.y, x1.y + x2.x) : make_float2(x1.x + x2.y, x2.x - x1.y);
     }
 }
-template <int N>
-__device__ __forceinline__ void pair_row(float2 (&v)[N / 32], int r, int lane, const float2 *__restrict__ t1,
-                                         const float2 *__restrict__ t2, const float2 *__restrict__ sp) {
-    PairRowRaw<N> w;
-    pair_row_load<N>(w, r, lane, t1, t2, sp);
-    pair_row_make<N>(v, w, lane);
-}
-
-// search_body for N = R x 32 >= 64: per template pair, each warp builds its
+// The multi-map queue's body for N = R x 32 >= 64: pattern p against template pairs
+// [pb, pe), smem_bytes<N>() of the group's shared memory; folds the item's best into
+// keys[p].  Per template pair, each warp builds its
 // rows of Z from the spectra straight into registers, transforms them
 // (warp_fft_core) and stores them once; after one barrier each warp loads its
 // columns, transforms them and keeps the running maxima of the real and
 // imaginary parts in registers (the surface is never written back); after a
 // second barrier thread 0 combines the warps' maxima.
-// PF: fetch the next row's spectra a row ahead (R x 6 more registers per
-// thread: for CTAs of at most 512 threads, whose register budget has room)
-template <int N, bool PF = true>
+// The next row's spectra are fetched a row ahead (R x 6 more registers per thread, which
+// the 512-thread queue CTAs have).
+template <int N>
 __device__ void search_body_reg(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, int p, int pb,
-                                int pe, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
-                                const int *__restrict__ cand, int kc, const Grp &g) {
+                                int pe, unsigned long long *__restrict__ keys, const Grp &g) {
     constexpr int LD = N + 1, HW = N / 2 + 1, R = N / 32;
     float2 *buf = reinterpret_cast<float2 *>(g.smem);
     float2 *twi = buf + N * LD;
@@ -256,36 +248,23 @@ __device__ void search_body_reg(const float2 *__restrict__ St, int T, const floa
     WarpFftTw<N> tw;
     tw.load(twi, lane);
     const float2 *sp = Sp + (size_t)p * N * HW;
-    const int n = cand ? kc : T;
     float best_v = -INFINITY;
     int best_t = -1;
     for (int pi = pb; pi < pe; ++pi) {
-        const int j1 = 2 * pi, j2 = min(j1 + 1, n - 1);
-        const int t1 = cand ? cand[(size_t)p * kc + j1] : j1;
-        const int t2 = cand ? cand[(size_t)p * kc + j2] : j2;
-        const float2 *s1 = St + (size_t)max(t1, 0) * N * HW, *s2 = St + (size_t)max(t2, 0) * N * HW;
+        const int t1 = 2 * pi, t2 = min(t1 + 1, T - 1);
+        const float2 *s1 = St + (size_t)t1 * N * HW, *s2 = St + (size_t)t2 * N * HW;
         // rows (the previous pair's column reads ended at its second barrier); the
         // spectra of the warp's next row are fetched before this row is transformed,
         // so their L2 latency overlaps the transform
-        if constexpr (PF) {
-            PairRowRaw<N> raw;
-            if (w < N) pair_row_load<N>(raw, w, lane, s1, s2, sp);
-            for (int r = w; r < N; r += nw) {
-                float2 v[R];
-                pair_row_make<N>(v, raw, lane);
-                if (r + nw < N) pair_row_load<N>(raw, r + nw, lane, s1, s2, sp);
-                warp_fft_core<N>(v, tw, lane);
+        PairRowRaw<N> raw;
+        if (w < N) pair_row_load<N>(raw, w, lane, s1, s2, sp);
+        for (int r = w; r < N; r += nw) {
+            float2 v[R];
+            pair_row_make<N>(v, raw, lane);
+            if (r + nw < N) pair_row_load<N>(raw, r + nw, lane, s1, s2, sp);
+            warp_fft_core<N>(v, tw, lane);
 #pragma unroll
-                for (int j = 0; j < R; ++j) buf[r * LD + warp_fft_out<N>(lane, j)] = v[j];
-            }
-        } else {
-            for (int r = w; r < N; r += nw) {
-                float2 v[R];
-                pair_row<N>(v, r, lane, s1, s2, sp);
-                warp_fft_core<N>(v, tw, lane);
-#pragma unroll
-                for (int j = 0; j < R; ++j) buf[r * LD + warp_fft_out<N>(lane, j)] = v[j];
-            }
+            for (int j = 0; j < R; ++j) buf[r * LD + warp_fft_out<N>(lane, j)] = v[j];
         }
         g.sync();
         // columns: maxima only
@@ -315,26 +294,15 @@ __device__ void search_body_reg(const float2 *__restrict__ St, int T, const floa
                 m1 = fmaxf(m1, red[i].x);
                 m2 = fmaxf(m2, red[i].y);
             }
-            if (t1 < 0) m1 = -INFINITY;
-            if (t2 < 0) m2 = -INFINITY;
-            if (t1 >= 0 && (m1 > best_v || (m1 == best_v && t1 < best_t))) { best_v = m1; best_t = t1; }
-            if (j2 != j1 && t2 >= 0 && (m2 > best_v || (m2 == best_v && t2 < best_t))) { best_v = m2; best_t = t2; }
-            if (peaks_all) {
-                peaks_all[(size_t)p * n + j1] = m1;
-                if (j2 != j1) peaks_all[(size_t)p * n + j2] = m2;
-            }
+            if (m1 > best_v || (m1 == best_v && t1 < best_t)) { best_v = m1; best_t = t1; }
+            if (t2 != t1 && (m2 > best_v || (m2 == best_v && t2 < best_t))) { best_v = m2; best_t = t2; }
         }
     }
     if (g.t == 0 && best_t >= 0) atomicMax(keys + p, pack_key(best_v, best_t));
 }
-template <int N, bool PF = true>
-__device__ void search_body_reg(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, int p, int pb,
-                                int pe, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
-                                const int *__restrict__ cand, int kc) {
-    search_body_reg<N, PF>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc, cta_group());
-}
 
-// search body with the whole surface in shared memory: per template pair the
+// search body with the whole surface in shared memory (slots: every template, or the
+// pattern's candidate list): per template pair the
 // full spectrum Z is built in shared memory, transformed by rows and by
 // columns with radix-2 butterfly line FFTs in shared memory, and scanned for
 // the maxima (any power-of-two N up to 64; blockDim-strided loops)
@@ -379,26 +347,6 @@ __device__ void search_body_smem(const float2 *__restrict__ St, int T, const flo
         }
     }
     if (g.t == 0 && best_t >= 0) atomicMax(keys + p, pack_key(best_v, best_t));
-}
-template <int N>
-__device__ void search_body_smem(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, int p, int pb,
-                                 int pe, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
-                                 const int *__restrict__ cand, int kc) {
-    search_body_smem<N>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc, cta_group());
-}
-
-// One work item: pattern p against slot pairs [pb, pe) (slots = all
-// templates, or the pattern's candidate list); smem_bytes<N>() of dynamic
-// shared memory; folds the item's best into keys[p].  N >= 64 takes
-// search_body_reg, smaller sides search_body_smem.
-template <int N, bool PF = true>
-__device__ void search_body(const float2 *__restrict__ St, int T, const float2 *__restrict__ Sp, int p, int pb,
-                            int pe, unsigned long long *__restrict__ keys, float *__restrict__ peaks_all,
-                            const int *__restrict__ cand, int kc) {
-    if constexpr (N >= 64)
-        search_body_reg<N, PF>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
-    else
-        search_body_smem<N>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
 }
 
 // dynamic shared memory of one search item: the N x (N + 1) surface, N

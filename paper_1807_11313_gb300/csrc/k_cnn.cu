@@ -562,27 +562,18 @@ __global__ void k_fallback_flags(const float *__restrict__ peak, const int *__re
     if ((threadIdx.x & 31) == 0 && m) atomicAdd(count, __popc(m));
 }
 
-// search mask (patterns without fallback are skipped as if degenerate) and
-// the seeds of the second refinement: library orientation of the best
-// template where a fallback happens, the current orientation elsewhere
+// search mask: patterns without fallback are skipped as if degenerate
 __global__ void k_fallback_mask(const int *__restrict__ degen, const int *__restrict__ fb, int P,
                                 int *__restrict__ mask) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < P) mask[p] = degen[p] || !fb[p];
 }
-__global__ void k_fallback_seeds(const int *__restrict__ fb, const int *__restrict__ best,
-                                 const double *__restrict__ lib_q, const double *__restrict__ cur, int P,
-                                 double *__restrict__ seeds) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const bool use = fb[p] && best[p] >= 0;
-    for (int i = 0; i < 4; ++i) seeds[4 * p + i] = use ? lib_q[4L * best[p] + i] : cur[4 * p + i];
-}
 
 // the fallback batch by pattern pairs (one block of 1024 threads): every
 // pair (2j, 2j + 1) with a flagged member, in order, at (2i, 2i + 1), so that
-// each pattern keeps the partner it shares a complex inverse transform with
-// in the pair-peak kernels; flag_c marks the flagged members (a last pair
+// each pattern keeps the partner it shares a complex transform with at the native
+// 160 px (k_prep_cplx, k_pair_peak; the other sides take one pattern at a time);
+// flag_c marks the flagged members (a last pair
 // without a second pattern repeats the first, unflagged); pairs[0] = count
 __global__ void __launch_bounds__(1024) k_fallback_list(const int *__restrict__ fb, int P, int *__restrict__ idx,
                                                         int *__restrict__ flag_c, int *__restrict__ pairs) {
@@ -940,12 +931,5 @@ cudaError_t launch_fallback_scatter(const int *idx, const int *flag_c, int n, co
                                     const int *it_c, double *q, float *peak, int *iters, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     k_fallback_scatter<<<(n + 255) / 256, 256, 0, st>>>(idx, flag_c, n, q_c, peak_c, it_c, q, peak, iters);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fallback_seeds(const int *fb, const int *best, const double *lib_q, const double *cur, int P,
-                                  double *seeds, cudaStream_t st) {
-    if (P <= 0) return cudaSuccess;
-    k_fallback_seeds<<<(P + 255) / 256, 256, 0, st>>>(fb, best, lib_q, cur, P, seeds);
     return cudaGetLastError();
 }

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kThreads) k_search_generic(const float2 *__res
     if (degen[p]) return;
     const int npairs = ((cand ? kc : T) + 1) / 2;
     const int pb = blockIdx.x * pairs_per_cta, pe = min(npairs, pb + pairs_per_cta);
-    search_body<N, true>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc);
+    search_body_smem<N>(St, T, Sp, p, pb, pe, keys, peaks_all, cand, kc, cta_group());
 }
 
 // N = 64 and 96: three register rounds on units of 64 and 192 threads: at 64 two
@@ -709,18 +709,17 @@ cudaError_t launch_search(int N, const float2 *St, int T, const float2 *Sp, cons
 }
 
 cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc, const float2 *Sp,
-                               const int *degen, int P, unsigned long long *keys, float *peaks, int num_sms,
-                               cudaStream_t st) {
+                               const int *degen, int P, unsigned long long *keys, int num_sms, cudaStream_t st) {
     if (P <= 0 || kc <= 0) return cudaSuccess;
     switch (N) {
-        case 16: return search_n<16>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
-        case 32: return search_n<32>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
-        case 64: return search_n<64>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
+        case 16: return search_n<16>(St, 0, Sp, degen, P, keys, nullptr, num_sms, st, cand, kc);
+        case 32: return search_n<32>(St, 0, Sp, degen, P, keys, nullptr, num_sms, st, cand, kc);
+        case 64: return search_n<64>(St, 0, Sp, degen, P, keys, nullptr, num_sms, st, cand, kc);
         case 128:   // St: the search layout, as for the search itself
-            return peaks ? cudaErrorInvalidValue : launch_search128_list(St, cand, kc, Sp, degen, P, keys, num_sms, st);
-        case 96: return search_n<96>(St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
+            return launch_search128_list(St, cand, kc, Sp, degen, P, keys, num_sms, st);
+        case 96: return search_n<96>(St, 0, Sp, degen, P, keys, nullptr, num_sms, st, cand, kc);
         case 160:
-        case 200: return launch_search_lines(N, St, 0, Sp, degen, P, keys, peaks, num_sms, st, cand, kc);
+        case 200: return launch_search_lines(N, St, 0, Sp, degen, P, keys, nullptr, num_sms, st, cand, kc);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -50,16 +50,16 @@ __device__ __forceinline__ void run_item(const MapDev &m, const WorkItem &w, con
             else if (m.body == kBodyOct)
                 rnd::search_body<64, false>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g);
             else
-                gen::search_body_reg<64>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g);
+                gen::search_body_reg<64>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, g);
             break;
-        case 96: gen::search_body_reg<96>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g); break;
+        case 96: gen::search_body_reg<96>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, g); break;
         case 128:
             if (m.body == kBodyRounds)   // whole CTAs only (phase 0)
                 s128::search_body<false>(m.Stp, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr);
             else
-                gen::search_body_reg<128>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g);
+                gen::search_body_reg<128>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, g);
             break;
-        case 160: gen::search_body_reg<160>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, nullptr, nullptr, 0, g); break;
+        case 160: gen::search_body_reg<160>(m.St, m.T, m.Sp, w.p, w.pb, w.pe, m.keys, g); break;
         default: break;   // not a queued side (the host never enqueues one)
     }
 }

@@ -196,8 +196,8 @@ __global__ void __launch_bounds__(kBgThreads) k_bg_cols(const float *__restrict_
     }
 }
 
-// ---- the same blur with the truncation radius R fixed at compile time (the
-// default sigma = N / 8 gives R = 3N / 8): the weights travel as a kernel
+// ---- the same blur at 256 x 256 with the truncation radius R fixed at compile time (the
+// default sigma = N / 8 gives R = 3N / 8; smaller sides: k_bg_norm): the weights travel as a kernel
 // parameter (constant bank, read as FMA operands of the unrolled taps) and
 // every thread slides one window over J consecutive outputs, so a loaded
 // pixel feeds up to J FMAs.
@@ -208,9 +208,9 @@ struct BgW {
 
 template <int N>
 struct BgShape {
-    static constexpr int J = N >= 64 ? 8 : N / 8;   // outputs per window
-    static constexpr int LANES = N < 32 ? N : 32;   // rows (row pass) / columns (column pass) per CTA
-    static constexpr int SPAN = N / 8;              // outputs of one warp along the blurred axis
+    static constexpr int J = 8;          // outputs per window
+    static constexpr int LANES = 32;     // rows (row pass) / columns (column pass) per CTA
+    static constexpr int SPAN = N / 8;   // outputs of one warp along the blurred axis
 };
 
 // row pass: LANES rows per CTA, lane = row, the 8 warps split the columns;
@@ -232,22 +232,20 @@ __global__ void __launch_bounds__(kBgThreads) k_bg_rows_t(const float *__restric
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane < S::LANES) {
-        const float *row = rows + lane * LD;
-        for (int c0 = warp * S::SPAN; c0 < (warp + 1) * S::SPAN; c0 += S::J) {
-            float acc[S::J];
+    const float *row = rows + lane * LD;
+    for (int c0 = warp * S::SPAN; c0 < (warp + 1) * S::SPAN; c0 += S::J) {
+        float acc[S::J];
 #pragma unroll
-            for (int j = 0; j < S::J; ++j) acc[j] = 0.f;
+        for (int j = 0; j < S::J; ++j) acc[j] = 0.f;
 #pragma unroll
-            for (int m = 0; m < 2 * R + S::J; ++m) {
-                const float v = row[c0 + m];
+        for (int m = 0; m < 2 * R + S::J; ++m) {
+            const float v = row[c0 + m];
 #pragma unroll
-                for (int j = 0; j < S::J; ++j)
-                    if (m - j >= 0 && m - j <= 2 * R) acc[j] = fmaf(W.w[m - j], v, acc[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < S::J; ++j) outs[lane * OLD + c0 + j] = acc[j];
+            for (int j = 0; j < S::J; ++j)
+                if (m - j >= 0 && m - j <= 2 * R) acc[j] = fmaf(W.w[m - j], v, acc[j]);
         }
+#pragma unroll
+        for (int j = 0; j < S::J; ++j) outs[lane * OLD + c0 + j] = acc[j];
     }
     __syncthreads();
     float *dst = tmp + (size_t)p * N * N + (size_t)r0 * N;
@@ -272,7 +270,6 @@ __global__ void __launch_bounds__(kBgThreads) k_bg_cols_t(const float *__restric
         strip[i] = __ldg(t + (size_t)min(max(q - R, 0), N - 1) * N + c);
     }
     __syncthreads();
-    if (lane >= L) return;
     const float *src = img + (size_t)p * img_stride + (size_t)oy * row_stride + ox + c0 + lane;
     float *dst = out + (size_t)p * N * N + c0 + lane;
     for (int q0 = warp * S::SPAN; q0 < (warp + 1) * S::SPAN; q0 += S::J) {

@@ -67,10 +67,9 @@ cudaError_t launch_prep_c256(const float *img, int P, const PrepArgs &a, float2 
                              const int *active, cudaStream_t st);
 
 // search over each pattern's candidate list cand [P][kc] (library indices, < 0 empty);
-// N = 128: St in the search layout, no peaks
+// N = 128: St in the search layout
 cudaError_t launch_search_list(int N, const float2 *St, const int *cand, int kc, const float2 *Sp,
-                               const int *degen, int P, unsigned long long *keys, float *peaks, int num_sms,
-                               cudaStream_t st);
+                               const int *degen, int P, unsigned long long *keys, int num_sms, cudaStream_t st);
 
 // BF16 zero-shift screen S[P][T] = A[P][K] . B[T][K]^T on tcgen05; err set on a timed-out wait
 cudaError_t launch_screen_tc(const void *A, int P, const void *B, int T, int K, float *S, int *err,
@@ -283,8 +282,6 @@ cudaError_t launch_fallback_seeds_list(const int *idx, const int *flag_c, const 
                                        const double *cur, int n, double *seeds, cudaStream_t st);
 cudaError_t launch_fallback_scatter(const int *idx, const int *flag_c, int n, const double *q_c, const float *peak_c,
                                     const int *it_c, double *q, float *peak, int *iters, cudaStream_t st);
-cudaError_t launch_fallback_seeds(const int *fb, const int *best, const double *lib_q, const double *cur, int P,
-                                  double *seeds, cudaStream_t st);
 
 // FP32 FMA rate probe (k_peak.cu): flops of one launch of the given shape
 cudaError_t launch_fma_rate(int blocks, int threads, int iters, float *sink, cudaStream_t st);
