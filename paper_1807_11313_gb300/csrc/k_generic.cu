@@ -331,15 +331,16 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
     }
     const CropStats csA = block_stats(a1, a2, xa0, N * N), csB = block_stats(b1, b2, xb0, N * N);
     bool badA = !ha || csA.bad, badB = !hb || csB.bad;
-    // ---- standardise and window (a degenerate crop becomes zeros)
+    // ---- standardise and window (a degenerate crop becomes zeros: its pixels may be NaN or
+    // infinite, and the two images share the transform)
     {
-        const float mA = csA.mean, iA = badA ? 0.f : csA.inv;
-        const float mB = csB.mean, iB = badB ? 0.f : csB.inv;
+        const float mA = csA.mean, iA = csA.inv;
+        const float mB = csB.mean, iB = csB.inv;
         for (int idx = tid; idx < N * N; idx += NT) {
             const int r = idx / N, c = idx - r * N;
             const float w = a.window ? 0.25f * (1.f - cospif(2.f * r / N)) * (1.f - cospif(2.f * c / N)) : 1.f;
             const float2 z = buf[r * LD + c];
-            buf[r * LD + c] = make_float2((z.x - mA) * iA * w, (z.y - mB) * iB * w);
+            buf[r * LD + c] = make_float2(badA ? 0.f : (z.x - mA) * iA * w, badB ? 0.f : (z.y - mB) * iB * w);
         }
     }
     __syncthreads();
@@ -419,8 +420,8 @@ __global__ void __launch_bounds__(kPrepCplxThreads, 1) k_prep_cplx(const float *
     for (int idx = tid; idx < N * N; idx += NT) {
         const int r = idx / N, c = idx - r * N;
         const float2 z = buf[r * LD + c];
-        if (ha) spatial[(size_t)pa * N * N + idx] = z.x * invn;
-        if (hb) spatial[(size_t)pb * N * N + idx] = z.y * invn;
+        if (ha) spatial[(size_t)pa * N * N + idx] = badA ? 0.f : z.x * invn;   // not the other image's rounding
+        if (hb) spatial[(size_t)pb * N * N + idx] = badB ? 0.f : z.y * invn;
     }
 }
 
