@@ -358,15 +358,16 @@ int xcf_nearest_disorientation(xcf_ctx *ctx, const double *qa, int32_t na, const
  * native rule).  Patterns are pre-processed per map, then every map up to
  * 160 x 160 is searched in ONE persistent launch (one 512-thread CTA per SM)
  * that takes (map, pattern, template range) work items of all sides from one
- * queue; 256 x 256 maps (thread-block clusters) and native 200 x 200 maps (one
- * template per pass through the real-output transform) run their own search
- * kernels in the same stream.  For each (detector side, library size) the
+ * queue; 256 x 256 maps (thread-block clusters) and native 200 x 200 maps (packed
+ * complex lines, one template at a time) run their own search kernels in the same
+ * stream.  For each (detector side, library size) the
  * search body and the work granularity are chosen by timing candidates on the
  * first call (cached in the context; see xcf_maps_get_tuning): the body is one
  * of the line-transform decompositions the queue has for that side,
  *   XCF_BODY_REG     rows and columns as warp-line transforms in registers,
  *                    N = R x 32 points (64, 96, 128, 160): R points per lane,
- *                    five 32-point lane stages by shuffles;
+ *                    five 32-point lane stages by shuffles (the only body at
+ *                    native 96 and 160, where xcf_index runs kernels of its own);
  *   XCF_BODY_ROUNDS  N = 128 only: three register rounds (16-point column
  *                    FFTs; radix 8 + radix 4; 32-point row FFTs) with two
  *                    shared-memory transposes (the kernel of xcf_index);
@@ -374,7 +375,8 @@ int xcf_nearest_disorientation(xcf_ctx *ctx, const double *qa, int32_t na, const
  *                    line transforms;
  *   XCF_BODY_OCT     N = 64 only: three register rounds (8-point column FFTs;
  *                    radix 8 x 2; 32-point row FFTs) of one template on a unit
- *                    of 64 threads (the kernel of xcf_index at N = 64);
+ *                    of 64 threads (the kernel of xcf_index at N = 64; the name
+ *                    is an earlier body's, of eight-lane groups);
  * the number of patterns a CTA searches side by side (1, 2 or 4 groups of
  * warps, each with its share of the shared memory, where the body fits), and
  * the granularity, the number of template pairs per work item (the whole

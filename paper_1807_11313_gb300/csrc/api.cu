@@ -1926,8 +1926,9 @@ const xcf_ctx::Tuning *tuned(const xcf_ctx *ctx, int N, int T) {
 // (and graph)
 bool queued_side(int N) { return N != 256 && N != 200; }
 
-// the body and grouping a side runs before (or without) tuning: the body of
-// its per-map kernel on whole CTAs
+// the body and grouping a side runs before (or without) tuning: whole CTAs with the
+// body of its per-map kernel, or where that has none in the queue (native 96 and 160)
+// the warp-line body
 int default_body(int N) { return N == 128 ? kBodyRounds : N == 64 ? kBodyOct : N < 64 ? kBodySmem : kBodyReg; }
 // whether G groups per CTA fit body b of side N (each group gets 1/G of the shared memory)
 bool groups_fit(int N, int b, int G) {

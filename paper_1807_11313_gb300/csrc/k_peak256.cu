@@ -8,7 +8,7 @@
 // neighbours are read from wherever they lie.
 //
 // What bounds it: latency (five cluster barriers per surface, 528 KB of spectra from
-// memory).  1,000 surfaces: 0.45 -> 0.21 ms against two surfaces per complex
+// memory).  1,000 surfaces: 0.45 -> 0.22 ms against two surfaces per complex
 // transform, rows first, one cluster of 256-thread CTAs per four SMs and the columns
 // around each maximum transformed again.
 #include "kernels.cuh"

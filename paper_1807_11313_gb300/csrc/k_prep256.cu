@@ -23,11 +23,12 @@
 // clusters of four interleave on their SMs (1,000 images with the filtered image
 // and without, five launches: 1.88 ms; one cluster of two CTAs of 512 threads:
 // 1.93).  Against row spectra [64][129] per CTA gathered column by column, one
-// cluster of four with 256 threads per SM: 0.75 -> 0.35 us per image over those
-// five launches (3.73 -> 1.75 ms), 0.26 without and 0.40 with the filtered image.
-// The barriers release this CTA's shared memory only: a full release waits for the
-// previous image's stores on their way to memory (0.271 -> 0.258 us).  Separate
-// kernels with and without the way back: no difference.
+// cluster of four with 256 threads per SM: 0.75 -> 0.36 us per image over those
+// five launches (3.73 -> 1.81 ms), 0.263 without and 0.422 with the filtered image.
+// The barriers that publish a CTA's own values release its shared memory only: a full
+// release at each waits for the previous image's stores on their way to memory (0.271
+// us without the filtered image).  At 128 registers (two CTAs per SM) 364 bytes per
+// thread spill.  Separate kernels with and without the way back: no difference.
 #include "kernels.cuh"
 #include "passes256.cuh"
 

@@ -21,12 +21,13 @@
 // gathered.
 //
 // What bounds it: sixteen warps go through the passes together, and the load
-// queue (64 global and 16 cluster loads per thread and template) fills in the
+// queue (64 global and 18 cluster loads per thread and template) fills in the
 // first and third; issue is active 42 %.  300 patterns x 1,018 templates: 53.6 ->
-// 38.9 ms (15.9 -> 22.1 TFLOP/s, 27 % of the FP32 peak) against template pairs on
-// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.49 ms.  A
-// full release at the barrier between the column and line passes costs 3 % of that.
-// Measured without gain: 16-byte template loads from an aligned copy of the
+// 39.5 ms (15.9 -> 21.8 TFLOP/s, 27 % of the FP32 peak) against template pairs on
+// clusters of four; the 32-candidate rescore of 1,000 patterns 5.42 -> 4.54 ms.  The
+// release after the gathers is 0.5 ms of the 39.5; a full one at the barrier between
+// the column and line passes too would be 3 % more.
+// Measured without gain (without the release after the gathers): 16-byte template loads from an aligned copy of the
 // library with half of the pattern in shared memory (41.3), the next template's
 // first values loaded a pass ahead (49.4: spills), 1,024 threads at 64 registers
 // (42.2), all gathers as cluster loads (41.6); two clusters of four CTAs per four SMs
@@ -299,7 +300,7 @@ cudaError_t launch_search_c256(const float2 *St, int T, const float2 *Sp, const 
     // 40.2 ms, part by part 38.9, whole items 39.7).  Against about four items per cluster
     // whatever the remainder, 2,000 templates: 10 patterns 3.25 -> 2.61 ms, 77: 24.6 ->
     // 19.9, 500: 136 -> 128; 32 candidates of 77 patterns 432 -> 402 us, of 1,000 4.65 ->
-    // 4.49 ms.
+    // 4.49 ms (each side before the release after the gathers, 1 to 2 % on top).
     int nchunks = 1;
     long least = -1;
     const int most = (int)std::min<long>(n, std::max<long>(64, 4L * ncl_max / P));
